@@ -139,7 +139,7 @@ void ff_params_default(ff_params *p);
 /*
  * Creates a context for p->n particles on p->device (Sec. 2 model, Sec. 3
  * schemes) and allocates its device memory: about 0.5 KB per particle in FP32
- * and 0.8 KB in FP64 (66 GB and 110 GB at n = 2^27), gradient buffers apart.
+ * (0.6 KB up to 106,496 particles) and 0.8 KB in FP64 (66 GB and 110 GB at n = 2^27), gradient buffers apart.
  * The tree's cell arrays start with room for 2 n + 8192 cells (gases, chains
  * and dense packings use 1.2 to 1.8 cells per particle).  A build that needs
  * more raises a device flag instead of writing past them; that step and the
@@ -253,7 +253,8 @@ ff_status ff_tune_traversal(ff_ctx *ctx, const int32_t *groups, int32_t ngroups,
  * single-precision walk (interaction counting off, no dipole-position terms),
  * its own compiled block shape: threads per block and the resident blocks per
  * SM the kernel's register budget is set for; other walks use their group's
- * default shape.  The traversal is persistent (as many blocks as fit), so the
+ * default shape, and the plain single-precision walk of up to 106,496 particles
+ * has one shape of its own whatever the schedule.  The traversal is persistent (as many blocks as fit), so the
  * shape trades registers per thread against resident warps.  Every schedule
  * gives bit-identical fields and forces (each lane decides and sums for its own
  * particle in depth-first order).  ff_schedule_info fills the three numbers

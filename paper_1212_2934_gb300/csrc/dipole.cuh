@@ -9,6 +9,26 @@ namespace ffk {
 __device__ __forceinline__ float dip_rsqrt(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double dip_rsqrt(double x) { return rsqrt(x); }
 
+__device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float pmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double pmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float padd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double padd(double a, double b) { return __dadd_rn(a, b); }
+
+// r^2 of a pair, each fused operation written out: every walk forms the same bits.
+template <typename R>
+__device__ __forceinline__ R pair_r2(R rx, R ry, R rz)
+{
+    return rfma(rz, rz, rfma(rx, rx, pmul(ry, ry)));
+}
+// a.b, likewise.
+template <typename R>
+__device__ __forceinline__ R pair_dot(R ax, R ay, R az, R bx, R by, R bz)
+{
+    return rfma(az, bz, rfma(ax, bx, pmul(ay, by)));
+}
+
 // Reduced dipolar field of u_j and force on u_k at separation r = rho_k - rho_j
 // (Sec. 2, reduced Eqs. h_dip and f_dip), accumulated:
 //   h += [3 r (u_j.r) - u_j r^2] / r^5
@@ -34,6 +54,71 @@ __device__ __forceinline__ void dipole(R rx, R ry, R rz, R r2, R ukx, R uky, R u
     fx += rx * cr + ukx * cuk + ujx * cuj;
     fy += ry * cr + uky * cuk + ujy * cuj;
     fz += rz * cr + ukz * cuk + ujz * cuj;
+}
+
+// The same with each fused operation written out, for the FP32 walks: every walk
+// that adds the same terms in the same order gives the same bits.
+template <typename R>
+__device__ __forceinline__ void walk_dipole(R rx, R ry, R rz, R r2, R ukx, R uky, R ukz, R ujx, R ujy,
+                                       R ujz, R& hx, R& hy, R& hz, R& fx, R& fy, R& fz)
+{
+    const R ir = dip_rsqrt(r2);
+    const R ir2 = pmul(ir, ir);
+    const R ir3 = pmul(ir2, ir);
+    const R ir5 = pmul(ir3, ir2);
+    const R ir7 = pmul(ir5, ir2);
+    const R bj = pair_dot(ujx, ujy, ujz, rx, ry, rz);
+    const R bk = pair_dot(ukx, uky, ukz, rx, ry, rz);
+    const R a = pair_dot(ujx, ujy, ujz, ukx, uky, ukz);
+    const R s3 = pmul(R(3), ir5);
+    const R cuk = pmul(s3, bj), cuj = pmul(s3, bk);  // cuk = 3 (u_j.r) / r^5 serves h and f
+    hx = padd(hx, rfma(rx, cuk, -pmul(ujx, ir3)));
+    hy = padd(hy, rfma(ry, cuk, -pmul(ujy, ir3)));
+    hz = padd(hz, rfma(rz, cuk, -pmul(ujz, ir3)));
+    const R cr = rfma(s3, a, -pmul(pmul(pmul(R(15), bk), bj), ir7));
+    fx = padd(fx, rfma(ujx, cuj, rfma(ukx, cuk, pmul(rx, cr))));
+    fy = padd(fy, rfma(ujy, cuj, rfma(uky, cuk, pmul(ry, cr))));
+    fz = padd(fz, rfma(ujz, cuj, rfma(ukz, cuk, pmul(rz, cr))));
+}
+
+// The terms of two sources (components .x and .y) for one target, two FP32
+// operations per instruction: walk_dipole()'s operations in its order, so
+// each source's terms have the same bits.  v = -u_j: with the moment's sign
+// turned, (-3 / r^5)(v.r) is 3 (u_j.r) / r^5 and every product below has
+// walk_dipole()'s value without an instruction spent on a sign.  The caller adds the
+// terms one source after the other (h += t, f += s).
+struct DipoleTerms2 {
+    float2 tx, ty, tz, sx, sy, sz;
+};
+__device__ __forceinline__ float2 dup2(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 pair_r2_2(float2 rx, float2 ry, float2 rz)
+{
+    return __ffma2_rn(rz, rz, __ffma2_rn(rx, rx, __fmul2_rn(ry, ry)));
+}
+__device__ __forceinline__ DipoleTerms2 dipole2(float2 rx, float2 ry, float2 rz, float2 ir,
+                                                float2 ukx, float2 uky, float2 ukz, float2 vx,
+                                                float2 vy, float2 vz)
+{
+    DipoleTerms2 o;
+    const float2 ir2 = __fmul2_rn(ir, ir);
+    const float2 ir3 = __fmul2_rn(ir2, ir);
+    const float2 ir5 = __fmul2_rn(ir3, ir2);
+    const float2 ir7 = __fmul2_rn(ir5, ir2);
+    const float2 bj = __ffma2_rn(vz, rz, __ffma2_rn(vx, rx, __fmul2_rn(vy, ry)));    // -u_j.r
+    const float2 bk = __ffma2_rn(ukz, rz, __ffma2_rn(ukx, rx, __fmul2_rn(uky, ry)));
+    const float2 a = __ffma2_rn(vz, ukz, __ffma2_rn(vx, ukx, __fmul2_rn(vy, uky)));  // -u_j.u_k
+    const float2 s3 = __fmul2_rn(dup2(-3.0f), ir5);
+    const float2 cuk = __fmul2_rn(s3, bj);
+    const float2 cuj = __fmul2_rn(s3, bk);  // -3 (u_k.r) / r^5
+    o.tx = __ffma2_rn(rx, cuk, __fmul2_rn(vx, ir3));
+    o.ty = __ffma2_rn(ry, cuk, __fmul2_rn(vy, ir3));
+    o.tz = __ffma2_rn(rz, cuk, __fmul2_rn(vz, ir3));
+    const float2 cr =
+        __ffma2_rn(s3, a, __fmul2_rn(__fmul2_rn(__fmul2_rn(dup2(15.0f), bk), bj), ir7));
+    o.sx = __ffma2_rn(vx, cuj, __ffma2_rn(ukx, cuk, __fmul2_rn(rx, cr)));
+    o.sy = __ffma2_rn(vy, cuj, __ffma2_rn(uky, cuk, __fmul2_rn(ry, cr)));
+    o.sz = __ffma2_rn(vz, cuj, __ffma2_rn(ukz, cuk, __fmul2_rn(rz, cr)));
+    return o;
 }
 
 // The same terms with u_k's part of the force kept as one scalar: adds
@@ -73,7 +158,7 @@ __device__ __forceinline__ void dipole_acc(R rx, R ry, R rz, R r2, R ukx, R uky,
 }
 
 // The traversal's pair terms: FP64 takes the form above with u_k factored out
-// (fewer FP64 operations, the scarce ones on this part); FP32 keeps dipole(),
+// (fewer FP64 operations, the scarce ones on this part); FP32 keeps dipole()'s,
 // whose extra operations measured no slower than the accumulator they save.
 // A pair at r2 = 0 adds nothing in either.
 __device__ __forceinline__ void walk_pair(float rx, float ry, float rz, float r2, float ukx,
@@ -81,7 +166,7 @@ __device__ __forceinline__ void walk_pair(float rx, float ry, float rz, float r2
                                           float& hx, float& hy, float& hz, float& fx, float& fy,
                                           float& fz, float&)
 {
-    if (r2 > 0.0f) dipole<float>(rx, ry, rz, r2, ukx, uky, ukz, ujx, ujy, ujz, hx, hy, hz, fx, fy, fz);
+    if (r2 > 0.0f) walk_dipole<float>(rx, ry, rz, r2, ukx, uky, ukz, ujx, ujy, ujz, hx, hy, hz, fx, fy, fz);
 }
 
 __device__ __forceinline__ void walk_pair(double rx, double ry, double rz, double r2, double ukx,

@@ -66,6 +66,7 @@ struct ff_ctx {
     void* q2 = nullptr;
     ffk::dvec4* mom_hi = nullptr;
     int* parent = nullptr;
+    int4* child = nullptr;       // children of each cell (contexts of up to kWarpWalkMax)
     int* arrive = nullptr;
     int64_t cap = 0;
 
@@ -223,6 +224,7 @@ ffk::Tree<R> tree_of(ff_ctx* c)
     t.lo = static_cast<ffk::vec4<R>*>(c->lo);
     t.sum = static_cast<ffk::vec4<R>*>(c->sum);
     t.parent = c->parent;
+    t.child = c->child;
     t.arrive = c->arrive;
     t.ncells = reinterpret_cast<int*>(c->off + c->n);
     t.cap = c->cap;
@@ -506,7 +508,7 @@ void free_all(ff_ctx* c)
 {
     void* ptrs[] = {c->keys[0], c->keys[1], c->vals[0], c->vals[1], c->radix_tmp, c->cnt, c->off,
                     c->scan_tmp, c->bbox, c->cell, c->mom, c->lo, c->sum, c->sum_hi, c->mom_hi,
-                    c->q1, c->q2, c->parent,
+                    c->q1, c->q2, c->parent, c->child,
                     c->arrive, c->h, c->f, c->esr, c->counts, c->work, c->partials, c->obs, c->obs_step, c->dstep, c->sys_of_pos, c->sys_start, c->sys_h, c->sys_lo,
                     c->sys_hi, c->sys_acc,
                     c->dflags, c->staging, c->e_cnt, c->e_base, c->e_total, c->g_pos, c->g_u,
@@ -556,12 +558,13 @@ int64_t initial_cells(int64_t n)
 ff_status alloc_cells(ff_ctx* c, int64_t cap)
 {
     void* olds[] = {c->cell, c->mom, c->lo, c->sum, c->sum_hi, c->mom_hi, c->q1, c->q2,
-                    c->parent, c->arrive};
+                    c->parent, c->child, c->arrive};
     for (void* q : olds)
         if (q) cudaFree(q);
     c->cell = c->mom = c->lo = c->sum = c->q1 = c->q2 = nullptr;
     c->sum_hi = c->mom_hi = nullptr;
     c->parent = c->arrive = nullptr;
+    c->child = nullptr;
     c->cap = 0;
     const size_t rec = c->rec;
     cudaError_t e = cudaSuccess;
@@ -581,6 +584,9 @@ ff_status alloc_cells(ff_ctx* c, int64_t cap)
         A(&c->q2, rec * cap);
     }
     A(&c->parent, sizeof(int) * cap);
+    // the shared walk of small single-precision contexts reads the children's table
+    if (!c->fp64 && !c->p.quadrupole && c->n <= ffk::kWarpWalkMax)
+        A(&c->child, 2 * sizeof(int4) * cap);
     A(&c->arrive, sizeof(int) * cap);
     if (e != cudaSuccess)
         return fail(c, FF_ENOMEM, "device allocation of %lld cells failed: %s", (long long)cap,

@@ -149,6 +149,9 @@ struct Tree {
     int* arrive;         // aggregation arrival counters
     int* ncells;         // device word: number of cells
     int64_t cap;         // allocated cells
+    int4* child;         // two per inner cell c: number of children, then the indices of the
+                         // second to the eighth (-1: none; the first is c + 1); null where
+                         // no walk reads it
     // dipole-position (quadrupole) terms about the centre, when enabled (else null):
     // q1 = (S_xx, S_yy, S_zz, S_xy), q2 = (S_xz, S_yz, m, 0), S the symmetric part of
     // sum (rho_i - c) (x) u_i and m its trace
@@ -380,6 +383,15 @@ template <typename R>
 void bh_field(const vec4<R>* pos, const vec4<R>* u, int64_t n, Tree<R> t, FieldParams<R> fp,
               vec4<R>* h, vec4<R>* f, R* esr, int4* counts, int* flags, int* work, int group,
               int sched, const uint32_t* off, Segs sg, cudaStream_t s);
+
+// The plain FP32 walk (no counts, no dipole-position terms) of contexts of up to
+// kWarpWalkMax particles: a warp per few particles (k_walk.cu), with the bits of
+// the one-lane walk.  Needs t.child; t.cap <= kWarpWalkCells (its source words hold 29-bit indices).
+constexpr int64_t kWarpWalkMax = 106496;
+constexpr int64_t kWarpWalkCells = int64_t(1) << 29;
+void warp_walk(const float4* pos, const float4* u, int64_t n, Tree<float> t,
+               FieldParams<float> fp, float4* h, float4* f, float* esr, int* flags, int* work,
+               const uint32_t* off, Segs sg, cudaStream_t s);
 
 // All-pairs sum (Sec. 3.1, Algorithm 1).
 template <typename R>

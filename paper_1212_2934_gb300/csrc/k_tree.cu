@@ -834,9 +834,13 @@ __global__ void k_aggregate(const vec4<R>* __restrict__ pos, const vec4<R>* __re
         int ch = par + 1;
         vec4<A> a = ldcg4(&ssum[ch]), b = ldcg4(&smom[ch]);
         sx = a.x; sy = a.y; sz = a.z; ux = b.x; uy = b.y; uz = b.z;
+        int kid[8] = {0, -1, -1, -1, -1, -1, -1, -1};
         ch = t.cell[ch].node.z;
         int kids = 1;
         while (ch < pn.z && kids < 8) {
+#pragma unroll
+            for (int k = 1; k < 8; ++k)
+                if (k == kids) kid[k] = ch;
             a = ldcg4(&ssum[ch]);
             b = ldcg4(&smom[ch]);
             sx = radd(sx, a.x);
@@ -851,6 +855,10 @@ __global__ void k_aggregate(const vec4<R>* __restrict__ pos, const vec4<R>* __re
         if (ch != pn.z || ++guard > kMaxLevel + 1) {
             atomicOr(flags, FLAG_AGGREGATE);
             break;
+        }
+        if (t.child) {
+            t.child[2 * (int64_t)par] = make_int4(kids, kid[1], kid[2], kid[3]);
+            t.child[2 * (int64_t)par + 1] = make_int4(kid[4], kid[5], kid[6], kid[7]);
         }
         c = par;
         nd = pn;
