@@ -632,8 +632,8 @@ __global__ void __launch_bounds__(kBhThreads, (bh_rec_min_blocks<R>())) k_bh_rec
     }
 }
 
-// All pairs: one thread per target; source records staged through shared
-// memory one block-sized tile at a time (Sec. 3.1, Algorithm 1).
+// All pairs in FP64: one thread per target; source records staged through
+// shared memory one block-sized tile at a time (Sec. 3.1, Algorithm 1).
 constexpr int kApThreads = 256;
 
 template <typename R>
@@ -698,6 +698,142 @@ __global__ void __launch_bounds__(kApThreads) k_ap(const vec4<R>* __restrict__ p
     h[k] = ho;
     f[k] = fo;
     if (esr) esr[k] = es;
+}
+
+// All pairs in single precision: a block serves T targets (a lane each, 32 / T
+// times over) and its warps share out the sources, 32 at a time, each warp (and
+// each group of T lanes in it) a batch of its own; the groups' sums are added in
+// a fixed order at the end.  One thread per target left the chip idle below
+// 150,000 targets (20,011: 79 blocks of 256 on 152 SMs).  Two sources go through
+// each FP32 instruction, their sums kept apart, and with the powers of 1/r outside
+// the brackets the last operation of each component is one fused multiply-add
+// into its sum: 41 instructions for two pairs, 82 cycles of the FP32 pipe, which
+// bounds the kernel.  Every 256 sources of a warp the running sums go to the
+// totals, so rounding grows with the square root of the two levels, not of n.
+// 16 targets a block below kApWide (n = 4,096 still gives 256 blocks); 32 above,
+// where staging a source for twice the targets saves 5 %.
+constexpr int kAp2Warps = 8;
+constexpr int kAp2Pair = 20;           // words per staged pair (14 used)
+constexpr int kAp2Stage = 16 * kAp2Pair + 4;
+constexpr int64_t kApWide = 65536;
+
+template <int T>
+__global__ void __launch_bounds__(32 * kAp2Warps, 2) k_ap2(const float4* __restrict__ pos,
+                                                           const float4* __restrict__ u, int n,
+                                                           FieldParams<float> fp,
+                                                           float4* __restrict__ h,
+                                                           float4* __restrict__ f,
+                                                           float* __restrict__ esr)
+{
+    constexpr int kGroups = 32 / T;         // groups of T lanes in a warp
+    constexpr int kPairs = 16 / kGroups;    // staged pairs of each
+    constexpr int kSums = 10;
+    __shared__ __align__(16) float sm[kAp2Warps * kAp2Stage];
+    static_assert(kAp2Warps * kAp2Stage >= kAp2Warps * 32 * kSums, "room for the partial sums");
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, grp = lane / T;
+    const int k = blockIdx.x * T + lane % T;
+    const float4 xk = pos[min(k, n - 1)], uk = u[min(k, n - 1)];
+    float* stage = sm + w * kAp2Stage;
+    // (the second group's pairs start 4 words on: other banks)
+    float* mine = stage + (lane >> 1) * kAp2Pair + (lane & 1) + ((lane >> 1) >= kPairs ? 4 : 0);
+    const float* own = stage + grp * (kPairs * kAp2Pair + 4);
+    const float2 kx = dup2(xk.x), ky = dup2(xk.y), kz = dup2(xk.z);
+    const float2 ux = dup2(uk.x), uy = dup2(uk.y), uz = dup2(uk.z);
+    const float2 zero = dup2(0.0f);
+    float2 thx = zero, thy = zero, thz = zero, tfx = zero, tfy = zero, tfz = zero;
+    float2 hx = zero, hy = zero, hz = zero, fx = zero, fy = zero, fz = zero;
+    float sx = 0.0f, sy = 0.0f, sz = 0.0f, es = 0.0f;
+    const float near2 = fp.include_sr ? fp.lj_rcut2_hi : 0.0f;
+    // past the end: no moment, far away
+    const float4 none = make_float4(1e18f, 1e18f, 1e18f, 0.0f);
+    int j = w * 32 + lane;
+    float4 c = j < n ? pos[j] : none, m = j < n ? u[j] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int base = w * 32, it = 1; base < n; base += 32 * kAp2Warps, ++it) {
+        __syncwarp();
+        mine[0] = -c.x;
+        mine[2] = -c.y;
+        mine[4] = -c.z;
+        mine[6] = m.x;
+        mine[8] = m.y;
+        mine[10] = m.z;
+        __syncwarp();
+        j += 32 * kAp2Warps;  // the next batch, under this one's arithmetic
+        c = j < n ? pos[j] : none;
+        m = j < n ? u[j] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        uint32_t close = 0u, one = 1u;
+        const float4* q = reinterpret_cast<const float4*>(own);
+#pragma unroll 2
+        for (int p = 0; p < kPairs; ++p, q += kAp2Pair / 4) {
+            const float4 q0 = q[0], q1 = q[1], q2 = q[2];
+            const float2 rx = __fadd2_rn(kx, make_float2(q0.x, q0.y));
+            const float2 ry = __fadd2_rn(ky, make_float2(q0.z, q0.w));
+            const float2 rz = __fadd2_rn(kz, make_float2(q1.x, q1.y));
+            const float2 vx = make_float2(q1.z, q1.w), vy = make_float2(q2.x, q2.y),
+                         vz = make_float2(q2.z, q2.w);
+            const float2 r2 = pair_r2_2(rx, ry, rz);
+            // the target itself, and coincident particles, add nothing
+            const float2 ir = make_float2(r2.x > 0.0f ? dip_rsqrt(r2.x) : 0.0f,
+                                          r2.y > 0.0f ? dip_rsqrt(r2.y) : 0.0f);
+            const float2 ir2 = __fmul2_rn(ir, ir);
+            const float2 ir3 = __fmul2_rn(ir2, ir);
+            const float2 p3 = __fmul2_rn(dup2(3.0f), ir2);
+            const float2 bj = __ffma2_rn(vz, rz, __ffma2_rn(vy, ry, __fmul2_rn(vx, rx)));
+            const float2 bk = __ffma2_rn(uz, rz, __ffma2_rn(uy, ry, __fmul2_rn(ux, rx)));
+            const float2 a = __ffma2_rn(vz, uz, __ffma2_rn(vy, uy, __fmul2_rn(vx, ux)));
+            // h += [3 r (u_j.r) / r^2 - u_j] / r^3
+            const float2 qh = __fmul2_rn(p3, bj);
+            const float2 nir3 = make_float2(-ir3.x, -ir3.y);
+            const float2 nqh = make_float2(-qh.x, -qh.y);
+            thx = __ffma2_rn(nir3, __ffma2_rn(rx, nqh, vx), thx);
+            thy = __ffma2_rn(nir3, __ffma2_rn(ry, nqh, vy), thy);
+            thz = __ffma2_rn(nir3, __ffma2_rn(rz, nqh, vz), thz);
+            // f += 3 / r^5 {r [u_j.u_k - 5 (u_k.r)(u_j.r) / r^2] + u_k (u_j.r) + u_j (u_k.r)}
+            const float2 g = __fmul2_rn(p3, ir3);
+            const float2 wv = __ffma2_rn(__fmul2_rn(dup2(-5.0f), ir2), __fmul2_rn(bj, bk), a);
+            tfx = __ffma2_rn(g, __ffma2_rn(rx, wv, __ffma2_rn(ux, bj, __fmul2_rn(vx, bk))), tfx);
+            tfy = __ffma2_rn(g, __ffma2_rn(ry, wv, __ffma2_rn(uy, bj, __fmul2_rn(vy, bk))), tfy);
+            tfz = __ffma2_rn(g, __ffma2_rn(rz, wv, __ffma2_rn(uz, bj, __fmul2_rn(vz, bk))), tfz);
+            if (r2.x < near2) close |= one;
+            if (r2.y < near2) close |= one << 1;
+            one <<= 2;
+        }
+        // LJ pairs within the cut, each lane its own
+        while (close != 0u) {
+            const int b = __ffs(close) - 1;
+            close &= close - 1u;
+            const float* st = own + (b >> 1) * kAp2Pair + (b & 1);
+            const float rx = xk.x + st[0], ry = xk.y + st[2], rz = xk.z + st[4];
+            lj<float>(fp, rx, ry, rz, pair_r2(rx, ry, rz), sx, sy, sz, es);
+        }
+        if ((it & 7) == 0) {
+            hx = __fadd2_rn(hx, thx); hy = __fadd2_rn(hy, thy); hz = __fadd2_rn(hz, thz);
+            fx = __fadd2_rn(fx, tfx); fy = __fadd2_rn(fy, tfy); fz = __fadd2_rn(fz, tfz);
+            thx = thy = thz = tfx = tfy = tfz = zero;
+        }
+    }
+    hx = __fadd2_rn(hx, thx); hy = __fadd2_rn(hy, thy); hz = __fadd2_rn(hz, thz);
+    fx = __fadd2_rn(fx, tfx); fy = __fadd2_rn(fy, tfy); fz = __fadd2_rn(fz, tfz);
+    __syncthreads();
+    float* r = sm + (w * 32 + lane) * kSums;
+    r[0] = hx.x + hx.y; r[1] = hy.x + hy.y; r[2] = hz.x + hz.y;
+    r[3] = fx.x + fx.y; r[4] = fy.x + fy.y; r[5] = fz.x + fz.y;
+    r[6] = sx; r[7] = sy; r[8] = sz; r[9] = es;
+    __syncthreads();
+    // component q of target t: the groups' sums in order
+    for (int e = threadIdx.x; e < T * kSums; e += 32 * kAp2Warps) {
+        const int t = e / kSums, q = e % kSums;
+        float v = 0.0f;
+        for (int g = 0; g < kAp2Warps * kGroups; ++g) v += sm[(g * T + t) * kSums + q];
+        sm[t * kSums + q] = v;  // (its own slot of group 0, read by no other sum)
+    }
+    __syncthreads();
+    if (threadIdx.x < T && k < n) {
+        const float* v = sm + threadIdx.x * kSums;
+        h[k] = make_float4(fp.dip_scale * v[0], fp.dip_scale * v[1], fp.dip_scale * v[2], 0.0f);
+        f[k] = make_float4(fp.dip_scale * v[3] + v[6], fp.dip_scale * v[4] + v[7],
+                           fp.dip_scale * v[5] + v[8], 0.0f);
+        if (esr) esr[k] = v[9];
+    }
 }
 
 }  // namespace
@@ -809,12 +945,23 @@ void bh_field_record(const vec4<R>* pos, const vec4<R>* u, int64_t n, Tree<R> t,
     counted();
 }
 
-template <typename R>
-void ap_field(const vec4<R>* pos, const vec4<R>* u, int64_t n, FieldParams<R> fp, vec4<R>* h,
-              vec4<R>* f, R* esr, cudaStream_t s)
+template <>
+void ap_field<double>(const dvec4* pos, const dvec4* u, int64_t n, FieldParams<double> fp, dvec4* h,
+                      dvec4* f, double* esr, cudaStream_t s)
 {
     const unsigned g = (unsigned)((n + kApThreads - 1) / kApThreads);
-    k_ap<R><<<g, kApThreads, 0, s>>>(pos, u, (int)n, fp, h, f, esr);
+    k_ap<double><<<g, kApThreads, 0, s>>>(pos, u, (int)n, fp, h, f, esr);
+    counted();
+}
+
+template <>
+void ap_field<float>(const float4* pos, const float4* u, int64_t n, FieldParams<float> fp,
+                     float4* h, float4* f, float* esr, cudaStream_t s)
+{
+    if (n < kApWide)
+        k_ap2<16><<<(unsigned)((n + 15) / 16), 32 * kAp2Warps, 0, s>>>(pos, u, (int)n, fp, h, f, esr);
+    else
+        k_ap2<32><<<(unsigned)((n + 31) / 32), 32 * kAp2Warps, 0, s>>>(pos, u, (int)n, fp, h, f, esr);
     counted();
 }
 
@@ -830,11 +977,6 @@ template void bh_field_record<float>(const float4*, const float4*, int64_t, Tree
 template void bh_field_record<double>(const dvec4*, const dvec4*, int64_t, Tree<double>,
                                       FieldParams<double>, dvec4*, dvec4*, double*, int4*, int*,
                                       int*, const uint32_t*, Segs, EntryPool, cudaStream_t);
-template void ap_field<float>(const float4*, const float4*, int64_t, FieldParams<float>, float4*,
-                              float4*, float*, cudaStream_t);
-template void ap_field<double>(const dvec4*, const dvec4*, int64_t, FieldParams<double>, dvec4*,
-                               dvec4*, double*, cudaStream_t);
-
 
 template <typename R, bool REC>
 void bh_vjp_launch(const vec4<R>* pos, int64_t n, Tree<R> t, FieldParams<R> fp, int* flags,
