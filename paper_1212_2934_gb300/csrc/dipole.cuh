@@ -123,52 +123,54 @@ __device__ __forceinline__ DipoleTerms2 dipole2(float2 rx, float2 ry, float2 rz,
 
 // The same terms with u_k's part of the force kept as one scalar: adds
 //   h += r cuk - u_j / r^3,   f += r cr + u_j cuj,   c += cuk,
-// cuk = 3 (u_j.r) / r^5, cuj = 3 (u_k.r) / r^5, cr = 3 (u_j.u_k) / r^5 - 15 (u_k.r)(u_j.r) / r^7,
+// cuk = 3 (u_j.r) / r^5, cuj = 3 (u_k.r) / r^5,
+// cr = 3 / r^5 [u_j.u_k - 5 (u_k.r)(u_j.r) / r^2],
 // so that the force on u_k is f + u_k c once every source has been added (u_k
-// is the same for all of them).  A pair at r2 = 0 adds nothing.
+// is the same for all of them).  A pair at r2 = 0 adds nothing.  Each operation
+// is written out: the counting and the plain walk give the same bits.
 template <typename R>
 __device__ __forceinline__ void dipole_acc(R rx, R ry, R rz, R r2, R ukx, R uky, R ukz, R ujx,
                                            R ujy, R ujz, R& hx, R& hy, R& hz, R& fx, R& fy,
                                            R& fz, R& c)
 {
     const R ir = r2 > R(0) ? dip_rsqrt(r2) : R(0);
-    const R ir2 = ir * ir;
-    const R ir3 = ir2 * ir;
-    const R ir5 = ir3 * ir2;
-    const R ir7 = ir5 * ir2;
-    const R bj = ujx * rx + ujy * ry + ujz * rz;
-    const R bk = ukx * rx + uky * ry + ukz * rz;
-    const R a = ujx * ukx + ujy * uky + ujz * ukz;
-    const R s3 = R(3) * ir5;
-    const R cuk = s3 * bj, cuj = s3 * bk;
-    hx += rx * cuk;
-    hy += ry * cuk;
-    hz += rz * cuk;
-    hx -= ujx * ir3;
-    hy -= ujy * ir3;
-    hz -= ujz * ir3;
-    const R cr = s3 * a - R(15) * bk * bj * ir7;
-    fx += rx * cr;
-    fy += ry * cr;
-    fz += rz * cr;
-    fx += ujx * cuj;
-    fy += ujy * cuj;
-    fz += ujz * cuj;
-    c += cuk;
+    const R ir2 = pmul(ir, ir);
+    const R ir3 = pmul(ir2, ir);
+    const R s3 = pmul(pmul(R(3), ir2), ir3);
+    const R bj = pair_dot(ujx, ujy, ujz, rx, ry, rz);
+    const R bk = pair_dot(ukx, uky, ukz, rx, ry, rz);
+    const R a = pair_dot(ujx, ujy, ujz, ukx, uky, ukz);
+    const R cuk = pmul(s3, bj), cuj = pmul(s3, bk);
+    const R cr = pmul(s3, rfma(pmul(R(-5), ir2), pmul(bj, bk), a));
+    hx = rfma(-ujx, ir3, rfma(rx, cuk, hx));
+    hy = rfma(-ujy, ir3, rfma(ry, cuk, hy));
+    hz = rfma(-ujz, ir3, rfma(rz, cuk, hz));
+    fx = rfma(ujx, cuj, rfma(rx, cr, fx));
+    fy = rfma(ujy, cuj, rfma(ry, cr, fy));
+    fz = rfma(ujz, cuj, rfma(rz, cr, fz));
+    c = padd(c, cuk);
 }
 
 // The traversal's pair terms: FP64 takes the form above with u_k factored out
 // (fewer FP64 operations, the scarce ones on this part); FP32 keeps dipole()'s,
-// whose extra operations measured no slower than the accumulator they save.
+// whose extra operations measured no slower than the accumulator they save, and
+// in the plain and counting walks with every operation written out (with the
+// dipole-position terms around it that order costs 4 %: left to the compiler).
 // A pair at r2 = 0 adds nothing in either.
+template <bool QUAD>
 __device__ __forceinline__ void walk_pair(float rx, float ry, float rz, float r2, float ukx,
                                           float uky, float ukz, float ujx, float ujy, float ujz,
                                           float& hx, float& hy, float& hz, float& fx, float& fy,
                                           float& fz, float&)
 {
-    if (r2 > 0.0f) walk_dipole<float>(rx, ry, rz, r2, ukx, uky, ukz, ujx, ujy, ujz, hx, hy, hz, fx, fy, fz);
+    if (!(r2 > 0.0f)) return;
+    if (QUAD)
+        dipole<float>(rx, ry, rz, r2, ukx, uky, ukz, ujx, ujy, ujz, hx, hy, hz, fx, fy, fz);
+    else
+        walk_dipole<float>(rx, ry, rz, r2, ukx, uky, ukz, ujx, ujy, ujz, hx, hy, hz, fx, fy, fz);
 }
 
+template <bool QUAD>
 __device__ __forceinline__ void walk_pair(double rx, double ry, double rz, double r2, double ukx,
                                           double uky, double ukz, double ujx, double ujy,
                                           double ujz, double& hx, double& hy, double& hz,

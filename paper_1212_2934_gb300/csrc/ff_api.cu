@@ -66,7 +66,7 @@ struct ff_ctx {
     void* q2 = nullptr;
     ffk::dvec4* mom_hi = nullptr;
     int* parent = nullptr;
-    int4* child = nullptr;       // children of each cell (contexts of up to kWarpWalkMax)
+    int4* child = nullptr;       // children of each cell (FP64, or up to kWarpWalkMax)
     int* arrive = nullptr;
     int64_t cap = 0;
 
@@ -584,8 +584,8 @@ ff_status alloc_cells(ff_ctx* c, int64_t cap)
         A(&c->q2, rec * cap);
     }
     A(&c->parent, sizeof(int) * cap);
-    // the shared walk of small single-precision contexts reads the children's table
-    if (!c->fp64 && !c->p.quadrupole && c->n <= ffk::kWarpWalkMax)
+    // the walks that serve several particles a warp read the children's table
+    if (!c->p.quadrupole && (c->fp64 || c->n <= ffk::kWarpWalkMax))
         A(&c->child, 2 * sizeof(int4) * cap);
     A(&c->arrive, sizeof(int) * cap);
     if (e != cudaSuccess)

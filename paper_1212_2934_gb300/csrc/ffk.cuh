@@ -393,6 +393,12 @@ void warp_walk(const float4* pos, const float4* u, int64_t n, Tree<float> t,
                FieldParams<float> fp, float4* h, float4* f, float* esr, int* flags, int* work,
                const uint32_t* off, Segs sg, cudaStream_t s);
 
+// The FP64 walk without dipole-position terms, with or without counts
+// (k_walk64.cu).  Needs t.child; t.cap <= kWarpWalkCells.
+void warp_walk64(const dvec4* pos, const dvec4* u, int64_t n, Tree<double> t,
+                 FieldParams<double> fp, dvec4* h, dvec4* f, double* esr, int4* counts, int* flags,
+                 int* work, const uint32_t* off, Segs sg, cudaStream_t s);
+
 // All-pairs sum (Sec. 3.1, Algorithm 1).
 template <typename R>
 void ap_field(const vec4<R>* pos, const vec4<R>* u, int64_t n, FieldParams<R> fp, vec4<R>* h,

@@ -194,7 +194,7 @@ __device__ __forceinline__ void bh_task(int task, const vec4<R>* __restrict__ po
                 // particle itself (centre and moment sum of one term are exact)
                 const R rx = xk.x - c.x, ry = xk.y - c.y, rz = xk.z - c.z;
                 const R r2 = pair_r2(rx, ry, rz);
-                walk_pair(rx, ry, rz, r2, uk.x, uk.y, uk.z, m.x, m.y, m.z, hx, hy, hz, fx, fy,
+                walk_pair<false>(rx, ry, rz, r2, uk.x, uk.y, uk.z, m.x, m.y, m.z, hx, hy, hz, fx, fy,
                               fz, ck);
                 if (acc) {
                     if (COUNT) ++nacc;
@@ -211,7 +211,7 @@ __device__ __forceinline__ void bh_task(int task, const vec4<R>* __restrict__ po
                         const R rx = xk.x - xj.x, ry = xk.y - xj.y, rz = xk.z - xj.z;
                         const R r2 = pair_r2(rx, ry, rz);
                         if (r2 > R(0)) {
-                            walk_pair(rx, ry, rz, r2, uk.x, uk.y, uk.z, uj.x, uj.y, uj.z, hx,
+                            walk_pair<false>(rx, ry, rz, r2, uk.x, uk.y, uk.z, uj.x, uj.y, uj.z, hx,
                                           hy, hz, fx, fy, fz, ck);
                             if (fp.include_sr) lj<R>(fp, rx, ry, rz, r2, sx, sy, sz, es);
                         }
@@ -350,7 +350,7 @@ __device__ __forceinline__ void bh_task1(int task, const vec4<R>* __restrict__ p
         if (acc || out1) {
             // the cell's pseudo-particle; for a one-particle leaf it is the
             // particle itself (centre and moment sum of one term are exact)
-            walk_pair(rx, ry, rz, r2, uk.x, uk.y, uk.z, m.x, m.y, m.z, hx, hy, hz, fx, fy, fz,
+            walk_pair<QUAD>(rx, ry, rz, r2, uk.x, uk.y, uk.z, m.x, m.y, m.z, hx, hy, hz, fx, fy, fz,
                           ck);
             if (REC) cw.put(i + (uint32_t)nd.x);
             if (QUAD && acc && r2 > R(0))
@@ -372,7 +372,7 @@ __device__ __forceinline__ void bh_task1(int task, const vec4<R>* __restrict__ p
                     const R rx = xk.x - xj.x, ry = xk.y - xj.y, rz = xk.z - xj.z;
                     const R r2 = pair_r2(rx, ry, rz);
                     if (r2 > R(0)) {
-                        walk_pair(rx, ry, rz, r2, uk.x, uk.y, uk.z, uj.x, uj.y, uj.z, hx, hy,
+                        walk_pair<QUAD>(rx, ry, rz, r2, uk.x, uk.y, uk.z, uj.x, uj.y, uj.z, hx, hy,
                                       hz, fx, fy, fz, ck);
                         if (fp.include_sr) lj<R>(fp, rx, ry, rz, r2, sx, sy, sz, es);
                     }
@@ -891,6 +891,17 @@ void bh_launch(const vec4<R>* pos, const vec4<R>* u, int64_t n, Tree<R> t, Field
 #undef FFK_SCHED
         }
     }
+    if constexpr (sizeof(R) == 8) {
+        // FP64: one walk for every lane group and schedule (trees of more cells than its
+        // source words can name, and dipole-position terms, keep the one-lane walk)
+        if (t.child && !t.q1 && t.cap <= kWarpWalkCells)
+            warp_walk64(pos, u, n, t, fp, h, f, esr, COUNT ? counts : nullptr, flags, work, off, sg, s);
+        else if (t.q1)
+            bh_launch_g<R, COUNT, 1, true>(pos, u, n, t, fp, h, f, esr, counts, flags, work, off, sg, s);
+        else
+            bh_launch_g<R, COUNT, 1>(pos, u, n, t, fp, h, f, esr, counts, flags, work, off, sg, s);
+        return;
+    } else {
     if (sched >= 1 && sched <= kNumSchedules) group = kSchedules[sched - 1].group;
     if (t.q1) {
         // the dipole-position terms are evaluated by the one-lane walk only
@@ -908,6 +919,7 @@ void bh_launch(const vec4<R>* pos, const vec4<R>* u, int64_t n, Tree<R> t, Field
         default: FFK_BH_CASE(32); break;
     }
 #undef FFK_BH_CASE
+    }
 }
 
 template <typename R>

@@ -24,28 +24,15 @@
 // warps to hide its loads and this one adds every source of a task in all of
 // its lanes (1784 of which a lane uses 813): the summing is bound by the FP32
 // pipe (84 % busy), the deciding by the latency of its rounds.
-#include "walk.cuh"
+#include "walk_stack.cuh"
 
 namespace ffk {
 
 namespace {
 
-constexpr int kStack = 512;   // pending cells per warp
 constexpr int kBatch = 64;    // sources summed together once this many are known
-constexpr int kList = 96;     // room for them: fewer than kBatch left, up to 32 new ones
 constexpr int kPairWords = 20;  // words per staged pair (16 used): fewer bank conflicts
 constexpr int kStageWords = 352;  // 16 staged pairs, or a round's mixed cells
-// above kStack - kStackSpare entries a round replaces one cell only: the
-// depth-first descent through the 22 levels then adds at most 7 a level
-constexpr int kStackSpare = 160;
-
-// source word: index | flags
-constexpr uint32_t kDone = 0x80000000u;      // decided: a source
-constexpr uint32_t kRun = 0x40000000u;       // an opened leaf of several particles
-constexpr uint32_t kLeafCell = 0x20000000u;  // source: a one-particle leaf
-constexpr uint32_t kParticle = 0x40000000u;  // source list only: a particle
-constexpr uint32_t kIndex = 0x1fffffffu;
-
 constexpr float kNormal = 1.1754944e-38f;  // smallest normal float
 
 // Block shape: 8 blocks of 2 warps an SM leave 128 registers a thread and 112 KB
@@ -55,8 +42,7 @@ constexpr int kWalkThreads = 64;
 constexpr int kWalkBlocks = 8;
 
 struct WarpShared {
-    uint2 stack[kStack];
-    uint2 list[kList];
+    WalkQueue q;
     float stage[kStageWords];
 };
 
@@ -152,7 +138,7 @@ __device__ __forceinline__ void sum_sources(WarpShared& w, int cnt, const Tree<f
             uint2 e = make_uint2(0u, 0u);
             float4 c = make_float4(0.0f, 0.0f, 0.0f, 0.0f), m = c;
             if (b + lane < cnt) {
-                e = w.list[b + lane];
+                e = w.q.list[b + lane];
                 const uint32_t i = e.x & kIndex;
                 const bool p = (e.x & kParticle) != 0u;
                 c = p ? pos[i] : t.cell[i].cen;
@@ -215,22 +201,11 @@ __device__ __forceinline__ int sum_full(WarpShared& w, int cnt, const Tree<float
     const int lane = threadIdx.x & 31, full = cnt & ~31;
     sum_sources(w, full, t, fp, near2, pos, u, k, a);
     uint2 e = make_uint2(0u, 0u);
-    if (lane < cnt - full) e = w.list[full + lane];
+    if (lane < cnt - full) e = w.q.list[full + lane];
     __syncwarp();
-    if (lane < cnt - full) w.list[lane] = e;
+    if (lane < cnt - full) w.q.list[lane] = e;
     __syncwarp();
     return cnt - full;
-}
-
-// Inclusive sum of v over the warp's lanes.
-__device__ __forceinline__ int warp_incscan(int v, int lane)
-{
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(kFull, v, o);
-        if (lane >= o) v += y;
-    }
-    return v;
 }
 
 __device__ __forceinline__ float warp_min(float v)
@@ -270,7 +245,7 @@ __device__ __forceinline__ void walk_task(WarpShared& w, int task, const float4*
     {
         const uint32_t am = __ballot_sync(kFull, active);
         if (!sg.of_pos) {
-            if (lane == 0) w.stack[0] = make_uint2(0u, am);
+            if (lane == 0) w.q.stack[0] = make_uint2(0u, am);
             top = 1;
         } else {
             const uint32_t sys = active ? sg.of_pos[k] : 0xffffffffu;
@@ -278,7 +253,7 @@ __device__ __forceinline__ void walk_task(WarpShared& w, int task, const float4*
             const bool lead = active && (mine & lt) == 0u;
             const uint32_t lm = __ballot_sync(kFull, lead);
             top = __popc(lm);
-            if (lead) w.stack[top - 1 - __popc(lm & lt)] = make_uint2(off[sg.start[sys]], mine);
+            if (lead) w.q.stack[top - 1 - __popc(lm & lt)] = make_uint2(off[sg.start[sys]], mine);
         }
     }
     int cnt = 0;
@@ -287,7 +262,7 @@ __device__ __forceinline__ void walk_task(WarpShared& w, int task, const float4*
         __syncwarp();
         const int seen = min(32, top);
         uint2 e = make_uint2(kDone, 0u);
-        if (lane < seen) e = w.stack[top - 1 - lane];
+        if (lane < seen) e = w.q.stack[top - 1 - lane];
         __syncwarp();
         const uint32_t runs = __ballot_sync(kFull, (e.x & kRun) != 0u);
         if (runs & 1u) {
@@ -299,7 +274,7 @@ __device__ __forceinline__ void walk_task(WarpShared& w, int task, const float4*
                 uint32_t mask = s < nd.y ? first.y : 0u;
                 if (s >= k0 && s < k0 + T) mask &= ~(1u << (s - k0));
                 const uint32_t keep = __ballot_sync(kFull, mask != 0u);
-                if (mask) w.list[cnt + __popc(keep & lt)] = make_uint2((uint32_t)s | kParticle, mask);
+                if (mask) w.q.list[cnt + __popc(keep & lt)] = make_uint2((uint32_t)s | kParticle, mask);
                 cnt += __popc(keep);
                 if (cnt >= kBatch) cnt = sum_full(w, cnt, t, fp, near2, pos, u, tg, a);
             }
@@ -309,7 +284,6 @@ __device__ __forceinline__ void walk_task(WarpShared& w, int task, const float4*
         const bool fresh = (e.x & kDone) == 0u;
         uint32_t acc = fresh ? 0u : e.y, open = 0u, own = 0u;
         uint32_t src = e.x & ~kDone;
-        int nkids = 0;
         bool mixed = false;
         int4 nd = make_int4(0, 0, 0, 0);
         float4 c, lo;
@@ -389,57 +363,7 @@ __device__ __forceinline__ void walk_task(WarpShared& w, int task, const float4*
                 open = e.y & ~got;
             }
         }
-        int4 ch0 = make_int4(0, 0, 0, 0), ch1 = ch0;
-        const bool run = open != 0u && (nd.w >> 8) != 0;
-        if (run) {
-            nkids = 1;
-        } else if (open != 0u) {
-            ch0 = t.child[2 * (int64_t)e.x];
-            ch1 = t.child[2 * (int64_t)e.x + 1];
-            nkids = ch0.x;
-        }
-        const int nout = (acc != 0u ? 1 : 0) + nkids;
-        int ex = warp_incscan(nout, lane);
-        int total = __shfl_sync(kFull, ex, 31), take = seen;
-        ex -= nout;
-        if (top - seen + total > kStack - kStackSpare) {
-            // only the cells whose replacements fit the stack (one always does)
-            const uint32_t fits = __ballot_sync(
-                kFull, lane < seen && top - lane - 1 + ex + nout <= kStack - kStackSpare);
-            take = max(1, fits == kFull ? 32 : __ffs(~fits) - 1);
-            if (take < seen) {
-                total = __shfl_sync(kFull, ex, take);
-                if (lane >= take) {
-                    acc = 0u;
-                    open = 0u;
-                }
-            }
-        }
-        // what comes before the first cell still to be looked into goes to the list
-        const uint32_t pm = __ballot_sync(kFull, open != 0u) | (runs & (kFull >> (32 - take)));
-        int emit = total;
-        if (pm != 0u) {
-            const int j0 = __ffs(pm) - 1;
-            emit = __shfl_sync(kFull, ex + ((acc != 0u && open != 0u) ? 1 : 0), j0);
-        }
-        top += total - emit - take;
-        int at = top - 1 - (ex - emit);
-        if (acc != 0u) {
-            if (ex < emit) w.list[cnt + ex] = make_uint2(src, acc);
-            else w.stack[at] = make_uint2(src | kDone, acc);
-            --at;
-        }
-        if (open != 0u) {
-            if (run) {
-                w.stack[at] = make_uint2(e.x | kDone | kRun, open);
-            } else {
-                w.stack[at] = make_uint2(e.x + 1u, open);
-                const int kid[7] = {ch0.y, ch0.z, ch0.w, ch1.x, ch1.y, ch1.z, ch1.w};
-#pragma unroll
-                for (int q = 1; q < 8; ++q)
-                    if (q < nkids) w.stack[at - q] = make_uint2((uint32_t)kid[q - 1], open);
-            }
-        }
+        const int emit = settle(w.q, cnt, lane, seen, runs, e, src, acc, open, nd.w, t.child, top);
         cnt += emit;
         if (cnt >= kBatch) {
             __syncwarp();

@@ -57,7 +57,7 @@ __device__ __forceinline__ float sigma2_minus_r2(const FieldParams<float>& fp, f
 __device__ __forceinline__ double sigma2_minus_r2(const FieldParams<double>& fp, double rx, double ry,
                                                   double rz)
 {
-    return fp.lj_sigma2 - (rx * rx + ry * ry + rz * rz);
+    return rsub(fp.lj_sigma2, pair_r2(rx, ry, rz));
 }
 
 // Printed LJ force (Sec. 2, Eq. LJ) inside the cut, and half the pair

@@ -1,11 +1,14 @@
-"""The shared walk of small single-precision contexts (csrc/k_walk.cu) against the counting walk.
+"""The walks that serve several particles a warp: of small single-precision contexts
+(csrc/k_walk.cu) against the counting walk, and of double precision (csrc/k_walk64.cu) against
+the oracle.
 
 Contexts of up to 106,496 particles without interaction counts take a walk in which a warp
 serves 8, 16 or 32 particles (n <= 8192, <= 26,624, above); with counts they take the one-lane
 walk.  Both add every particle's sources in the same order with the same operations, so fields
 and forces agree bit for bit, over the edges of the task sizes, leaves of several particles,
 LJ on and off, opening angles from 0 (every cell opened) to 0.9, tasks that span several
-systems, and coincident particles; the energies (sums of the same terms) agree too.
+systems, and coincident particles.  The double-precision walk is held to the repository's 1e-10
+and to exact interaction counts over the same options.
 """
 import numpy as np
 import pytest
@@ -33,14 +36,14 @@ def _gas(n, seed):
     return ((q + rng.uniform(-0.16, 0.16, (n, 3))) * 1.5).astype(np.float32), u.astype(np.float32)
 
 
-def _both(ff, pos, u, theta, sizes=None, **kw):
+def _both(ff, pos, u, theta, sizes=None, dtype=np.float32, **kw):
     out = []
     for count in (0, 1):
         ctx = ff.ff_create(ff.ff_params_default(n=len(pos), count_interactions=count, **kw))
         if sizes is not None:
             ff.ff_set_systems(ctx, sizes)
         ff.ff_set_particles(ctx, pos, u)
-        out.append(ff.ff_dipolar_field(ctx, ff.FF_ALGO_BH, theta, True, dtype=np.float32))
+        out.append(ff.ff_dipolar_field(ctx, ff.FF_ALGO_BH, theta, True, dtype=dtype))
     return out
 
 
@@ -82,3 +85,52 @@ def test_coincident_particles_and_flat_systems(ff):
     line[:, 0] = np.arange(3000) * 1.25
     (hp, fp), (hc, fc) = _both(ff, line, u[:3000], 0.5)
     assert np.array_equal(hp, hc) and np.array_equal(fp, fc)
+
+
+@pytest.mark.parametrize("theta", [0.0, 0.3, 0.9])
+@pytest.mark.parametrize("leaf_max", [1, 5, 64])
+@pytest.mark.parametrize("lj", [0.0, 1.0])
+def test_fp64_matches_oracle(ff, theta, leaf_max, lj):
+    import oracle
+    from conftest import rel_err
+
+    for n in (1, 7, 8, 9, 1501):
+        pos, u = _gas(n, 40 + n)
+        # off the single-precision grid, far from the origin
+        pos = pos.astype(np.float64) * (1.0 + 1e-9) + np.array([1000.0, -300.0, 7.0]) / 3.0
+        u = u.astype(np.float64)
+        (hp, fp), (hc, fc) = [(a, b) for a, b in _both(ff, pos, u, theta, precision="f64",
+                                                      leaf_max=leaf_max, lj_eps=lj,
+                                                      dtype=np.float64)]
+        assert np.array_equal(hp, hc) and np.array_equal(fp, fc)
+        if n == 1:
+            assert not hp.any() and not fp.any()
+            continue
+        ref = oracle.bh(pos, u, theta, leaf_max, "f64", 1.0, lj, 1.0, 2.5, True)
+        assert rel_err(hp, ref["h"]).max() <= 1e-10
+        assert rel_err(fp, ref["f"]).max() <= 1e-10
+        ctx = ff.ff_create(ff.ff_params_default(n=n, precision="f64", leaf_max=leaf_max,
+                                                lj_eps=lj, count_interactions=1))
+        ff.ff_set_particles(ctx, pos, u)
+        ff.ff_dipolar_field(ctx, ff.FF_ALGO_BH, theta, True)
+        acc, pairs, opened = ff.ff_get_counts(ctx)
+        assert np.array_equal(acc, ref["nacc"]) and np.array_equal(pairs, ref["npair"])
+        assert np.array_equal(opened, ref["nopen"])
+
+
+def test_fp64_tasks_spanning_systems(ff):
+    rng = np.random.default_rng(5)
+    sizes = [int(k) for k in rng.integers(1, 30, 200)]
+    parts = [_gas(k, i) for i, k in enumerate(sizes)]
+    pos = np.concatenate([p for p, _ in parts]).astype(np.float64)
+    u = np.concatenate([q for _, q in parts]).astype(np.float64)
+    (hp, fp), (hc, fc) = _both(ff, pos, u, 0.5, sizes=sizes, precision="f64", dtype=np.float64)
+    assert np.array_equal(hp, hc) and np.array_equal(fp, fc)
+    # each system alone gives the same bits: a particle's sums depend on its own sources
+    off = 0
+    for k, (p, q) in list(zip(sizes, parts))[:25]:
+        ctx = ff.ff_create(ff.ff_params_default(n=k, precision="f64"))
+        ff.ff_set_particles(ctx, p.astype(np.float64), q.astype(np.float64))
+        h, f = ff.ff_dipolar_field(ctx, ff.FF_ALGO_BH, 0.5, True)
+        assert np.array_equal(h, hp[off:off + k]) and np.array_equal(f, fp[off:off + k])
+        off += k
