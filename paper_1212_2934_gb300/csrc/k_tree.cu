@@ -298,6 +298,225 @@ __global__ void __launch_bounds__(kOsThreads, os_min_blocks<K>()) k_os_scatter(
     }
 }
 
+// ------------------------------------------------------- cluster key sort
+// The whole 64-bit key sort of up to 32,768 keys in one launch: a cluster of 1 to
+// 16 blocks keeps the (key, value) pairs in shared memory for all eight passes,
+// one or two pairs a thread.  A pass ranks each warp's consecutive keys in rounds
+// of 32 (as k_os_scatter does), exchanges the blocks' digit counts through
+// distributed shared memory, and sends every key to its place in the cluster's
+// shared memory.  What bounds a sort of this size is the latency of its passes: as
+// eight launches with a look-back between tiles they took 11 to 14 us each; here a
+// pass has two hardware cluster barriers instead and touches no global memory.
+// Stable, the same digits: the same order as the one-sweep sort.  Measured on
+// GB300, one-sweep -> this: n = 1,000 95 -> 27 us; 4,096 95 -> 36; 16,384
+// 111 -> 50; 32,768 113 -> 71.  With four pairs a thread 65,536 keys took 115 us
+// and with eight 131,072 took 199 us, the one-sweep sort 115 and 122: a block's
+// own share of a pass then costs more than the launch it saves.
+constexpr int kCsThreads = 1024;
+constexpr int kCsMaxBlocks = 16;
+constexpr int64_t kClusterSortMax = (int64_t)kCsThreads * 2 * kCsMaxBlocks;
+
+template <int ITEMS>
+struct ClusterSort {
+    static constexpr int kBlock = kCsThreads * ITEMS;
+    uint64_t key[kBlock];
+    uint32_t val[kBlock];
+    uint16_t wcnt[kCsThreads / 32][kRadixBins];  // per-warp digit counts, then prefixes
+    uint32_t cnt[kRadixBins];                    // the block's count of each digit
+    uint32_t start[kRadixBins];                  // where its keys of the digit go
+};
+
+// Address of a word of this block's shared memory in block `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank)
+{
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
+                 ::: "memory");
+}
+
+template <int ITEMS>
+__global__ void __launch_bounds__(kCsThreads, 1) k_cluster_sort(uint64_t* __restrict__ keys,
+                                                                uint32_t* __restrict__ vals, int n)
+{
+    extern __shared__ __align__(16) unsigned char cs_smem[];
+    constexpr int kBlock = ClusterSort<ITEMS>::kBlock;
+    ClusterSort<ITEMS>& sh = *reinterpret_cast<ClusterSort<ITEMS>*>(cs_smem);
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+    uint32_t rank, blocks;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(blocks));
+    const int base = (int)rank * kBlock;
+    const int mine = max(0, min(kBlock, n - base));
+    uint64_t key[ITEMS];
+    uint32_t val[ITEMS], pos[ITEMS];
+    const int e0 = w * 32 * ITEMS + lane;  // this thread's elements: e0 + 32 r
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const int e = e0 + 32 * r;
+        if (e < mine) {
+            key[r] = keys[base + e];
+            val[r] = vals[base + e];
+        }
+    }
+    for (int pass = 0; pass < 8; ++pass) {
+        const int shift = pass * kRadixBits;
+#pragma unroll
+        for (int j = 0; j < kRadixBins / 32; ++j) sh.wcnt[w][lane + 32 * j] = 0;
+        if (pass) {
+#pragma unroll
+            for (int r = 0; r < ITEMS; ++r) {
+                const int e = e0 + 32 * r;
+                if (e < mine) {
+                    key[r] = sh.key[e];
+                    val[r] = sh.val[e];
+                }
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < ITEMS; ++r) {
+            const bool valid = e0 + 32 * r < mine;
+            const uint32_t d =
+                valid ? (uint32_t)(key[r] >> shift) & (kRadixBins - 1) : (uint32_t)kRadixBins;
+            const uint32_t peers = __match_any_sync(kFull, d);
+            const uint32_t before = valid ? sh.wcnt[w][d] : 0u;
+            pos[r] = before + __popc(peers & lt);
+            __syncwarp();
+            if (valid && (peers & lt) == 0)
+                sh.wcnt[w][d] = (uint16_t)(before + __popc(peers));
+            __syncwarp();
+        }
+        __syncthreads();
+        // thread t owns digit t: prefixes over the warps, the block's count
+        if (t < kRadixBins) {
+            uint32_t c = 0;
+#pragma unroll 8
+            for (int ww = 0; ww < kCsThreads / 32; ++ww) {
+                const uint32_t v = sh.wcnt[ww][t];
+                sh.wcnt[ww][t] = (uint16_t)c;
+                c += v;
+            }
+            sh.cnt[t] = c;
+        }
+        // every block's counts are out, and its keys in registers
+        cluster_barrier();
+        uint32_t total = 0, before = 0;
+        if (t < kRadixBins) {
+            for (uint32_t b = 0; b < blocks; ++b) {
+                uint32_t v;
+                asm volatile("ld.shared::cluster.u32 %0, [%1];"
+                             : "=r"(v) : "r"(cluster_addr(&sh.cnt[t], b)));
+                if (b < rank) before += v;
+                total += v;
+            }
+        }
+        // digit starts: an exclusive sum over the 256 digits (the first eight warps)
+        __shared__ uint32_t ws[kRadixBins / 32];
+        uint32_t x = total;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(kFull, x, o);
+            if (lane >= o) x += y;
+        }
+        if (t < kRadixBins && lane == 31) ws[w] = x;
+        __syncthreads();
+        if (t < kRadixBins) {
+            uint32_t pre = 0;
+            for (int q = 0; q < w; ++q) pre += ws[q];
+            sh.start[t] = pre + x - total + before;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < ITEMS; ++r) {
+            if (e0 + 32 * r < mine) {
+                const uint32_t d = (uint32_t)(key[r] >> shift) & (kRadixBins - 1);
+                const uint32_t g = sh.start[d] + sh.wcnt[w][d] + pos[r];
+                const uint32_t b = g / kBlock, slot = g % kBlock;
+                asm volatile("st.shared::cluster.u64 [%0], %1;"
+                             ::"r"(cluster_addr(&sh.key[slot], b)), "l"(key[r]) : "memory");
+                asm volatile("st.shared::cluster.u32 [%0], %1;"
+                             ::"r"(cluster_addr(&sh.val[slot], b)), "r"(val[r]) : "memory");
+            }
+        }
+        cluster_barrier();
+    }
+    for (int e = t; e < mine; e += kCsThreads) {
+        keys[base + e] = sh.key[e];
+        vals[base + e] = sh.val[e];
+    }
+}
+
+cudaLaunchConfig_t cluster_config(int blocks, size_t smem, cudaLaunchAttribute* at, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = (unsigned)blocks;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kCsThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+// Sorts n keys in one cluster of 1, 2, 4, 8 or 16 blocks; false where the device
+// takes no such cluster (asked once per device).
+template <int ITEMS>
+bool cluster_sort_items(uint64_t* keys, uint32_t* vals, int64_t n, cudaStream_t s)
+{
+    constexpr int kDevs = 64;
+    static std::mutex mu;
+    static int most[kDevs];  // 0: not asked yet, else 1 + the largest cluster
+    const auto kern = k_cluster_sort<ITEMS>;
+    cudaLaunchAttribute at;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= kDevs) return false;
+    int b = 1;
+    while ((int64_t)b * kCsThreads * ITEMS < n) b *= 2;
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        if (most[dev] == 0) {
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(ClusterSort<ITEMS>));
+            cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            int best = 0;
+            for (int q = 1; q <= kCsMaxBlocks; q *= 2) {
+                const cudaLaunchConfig_t cfg =
+                    cluster_config(q, sizeof(ClusterSort<ITEMS>), &at, nullptr);
+                int active = 0;
+                if (cudaOccupancyMaxActiveClusters(&active, kern, &cfg) == cudaSuccess && active >= 1)
+                    best = q;
+                else
+                    cudaGetLastError();  // a size the device does not take is no error
+            }
+            most[dev] = 1 + best;
+        }
+        if (b > most[dev] - 1) return false;
+    }
+    const cudaLaunchConfig_t cfg = cluster_config(b, sizeof(ClusterSort<ITEMS>), &at, s);
+    if (cudaLaunchKernelEx(&cfg, kern, keys, vals, (int)n) != cudaSuccess) {
+        cudaGetLastError();  // the one-sweep sort takes over
+        return false;
+    }
+    counted();
+    return true;
+}
+
+bool cluster_sort(uint64_t* keys, uint32_t* vals, int64_t n, cudaStream_t s)
+{
+    if (n <= kCsThreads * kCsMaxBlocks) return cluster_sort_items<1>(keys, vals, n, s);
+    return cluster_sort_items<2>(keys, vals, n, s);
+}
+
 // ------------------------------------------------------- bbox and keys
 __device__ __forceinline__ long long enc(float x)
 {
@@ -961,6 +1180,8 @@ template bool radix_sort_pairs_passes<uint32_t>(uint32_t*, uint32_t*, uint32_t*,
 void radix_sort_pairs(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n,
                       uint32_t* tmp, int* flags, cudaStream_t s)
 {
+    // few keys: one launch of a cluster (kClusterSortMax)
+    if (n > 1 && n <= kClusterSortMax && cluster_sort(k0, v0, n, s)) return;
     // eight passes: the sorted data are back in (k0, v0)
     os_sort<uint64_t>(k0, v0, k1, v1, n, tmp, 8, flags, s, nullptr);
 }
