@@ -66,7 +66,8 @@ struct ff_ctx {
     void* q2 = nullptr;
     ffk::dvec4* mom_hi = nullptr;
     int* parent = nullptr;
-    int4* child = nullptr;       // children of each cell (FP64, or up to kWarpWalkMax)
+    int4* child = nullptr;       // children of each cell (FP64, up to kWarpWalkMax, or
+    bool need_child = false;     //   a single-precision context that takes gradients)
     int* arrive = nullptr;
     int64_t cap = 0;
 
@@ -126,6 +127,9 @@ struct ff_ctx {
     int64_t r_cap = 0;
     bool tree_valid = false;     // a Barnes-Hut tree of some state exists
     bool counts_valid = false;
+    bool counts_lazy = false;    // not recorded, but the last evaluation (below) can be counted
+    double lazy_theta = 0.0;     //   again: after a gradient on the shared walk
+    int lazy_sr = 0;
 
     // batched ensembles (ff_set_systems); nsys = 0: one system with the context's field and box
     int nsys = 0;
@@ -366,6 +370,33 @@ struct LaunchTally {
     }
 };
 
+// Whether the gradient's recording walk is the shared one (k_walk.cu), which
+// writes each task's records; else the one-lane walk writes each particle's list.
+bool shared_records(const ff_ctx* c)
+{
+    // a context that counts keeps the counting walk
+    return !c->fp64 && !c->p.count_interactions && c->child && c->cap <= ffk::kWarpWalkCells;
+}
+
+// The recording walk on the current tree.
+template <typename R>
+void record_walk(ff_ctx* c, double theta, int include_sr, const ffk::EntryPool& pool)
+{
+    Buffers& b = c->st[c->cur];
+    const ffk::FieldParams<R> fp = field_params<R>(c, theta, include_sr);
+    if constexpr (sizeof(R) == 4) {
+        if (shared_records(c)) {
+            ffk::warp_walk_record(V<R>(b.pos), V<R>(b.u), c->n, tree_of<R>(c), fp, V<R>(c->h),
+                                  V<R>(c->f), static_cast<R*>(c->esr), c->counts, c->t_cnt,
+                                  c->dflags, c->work, c->off, segs_of(c), pool, c->stream);
+            return;
+        }
+    }
+    ffk::bh_field_record<R>(V<R>(b.pos), V<R>(b.u), c->n, tree_of<R>(c), fp, V<R>(c->h), V<R>(c->f),
+                            static_cast<R*>(c->esr), c->counts, c->dflags, c->work, c->off,
+                            segs_of(c), pool, c->stream);
+}
+
 // Sort the state into Morton order (the other buffer), build and aggregate
 // the tree, traverse.  h, f, esr (and counts) end in sorted order.
 template <typename R>
@@ -412,10 +443,7 @@ ff_status eval_bh(ff_ctx* c, double theta, int include_sr, bool force_counts = f
     if (field) {
         StageTimer st(c, S_FIELD);
         if (pool)
-            ffk::bh_field_record<R>(V<R>(b.pos), V<R>(b.u), n, t,
-                                    field_params<R>(c, theta, include_sr), V<R>(c->h), V<R>(c->f),
-                                    static_cast<R*>(c->esr), c->counts, c->dflags, c->work, c->off,
-                                    segs_of(c), *pool, s);
+            record_walk<R>(c, theta, include_sr, *pool);
         else
             ffk::bh_field<R>(V<R>(b.pos), V<R>(b.u), n, t, field_params<R>(c, theta, include_sr),
                              V<R>(c->h), V<R>(c->f), static_cast<R*>(c->esr),
@@ -425,8 +453,26 @@ ff_status eval_bh(ff_ctx* c, double theta, int include_sr, bool force_counts = f
     }
     FF_LAUNCHED(c);
     c->tree_valid = true;
-    c->counts_valid = field && (c->p.count_interactions != 0 || force_counts || pool);
+    const bool lists = pool && !shared_records(c);  // the counting walk wrote them
+    c->counts_valid = field && (c->p.count_interactions != 0 || (force_counts && !pool) || lists);
+    c->counts_lazy = field && pool && !lists;
+    c->lazy_theta = theta;
+    c->lazy_sr = include_sr;
     return FF_OK;
+}
+
+// The interaction counts of a gradient's evaluation, whose walk does not split
+// its sources into cells and pairs: the counting walk on the same tree.
+template <typename R>
+void count_again(ff_ctx* c)
+{
+    Buffers& b = c->st[c->cur];
+    ffk::bh_field<R>(V<R>(b.pos), V<R>(b.u), c->n, tree_of<R>(c),
+                     field_params<R>(c, c->lazy_theta, c->lazy_sr), V<R>(c->h), V<R>(c->f),
+                     static_cast<R*>(c->esr), c->counts, c->dflags, c->work, traverse_group(c),
+                     c->sched, c->off, segs_of(c), c->stream);
+    c->counts_lazy = false;
+    c->counts_valid = true;
 }
 
 template <typename R>
@@ -585,7 +631,7 @@ ff_status alloc_cells(ff_ctx* c, int64_t cap)
     }
     A(&c->parent, sizeof(int) * cap);
     // the walks that serve several particles a warp read the children's table
-    if (!c->p.quadrupole && (c->fp64 || c->n <= ffk::kWarpWalkMax))
+    if (!c->p.quadrupole && (c->fp64 || c->n <= ffk::kWarpWalkMax || c->need_child))
         A(&c->child, 2 * sizeof(int4) * cap);
     A(&c->arrive, sizeof(int) * cap);
     if (e != cudaSuccess)
@@ -594,6 +640,7 @@ ff_status alloc_cells(ff_ctx* c, int64_t cap)
     c->cap = cap;
     c->tree_valid = false;
     c->counts_valid = false;
+    c->counts_lazy = false;
     return FF_OK;
 }
 
@@ -808,10 +855,25 @@ ff_status grow(ff_ctx* c, T** p, size_t count)
     return FF_OK;
 }
 
+// Slots of the record buffers: one per entry while lists are merged there, one
+// per record where they only serve the record sort.
+ff_status grow_slots(ff_ctx* c, int64_t need)
+{
+    ff_status st;
+    if (need <= c->e_cap) return FF_OK;
+    const int64_t cap = need + need / 8 + 1024;
+    if ((st = grow(c, &c->rs_key, cap)) != FF_OK) return st;
+    if ((st = grow(c, &c->rs_mask, cap)) != FF_OK) return st;
+    if ((st = grow(c, &c->e_tmp, ffk::radix_tmp_words(cap))) != FF_OK) return st;
+    c->e_cap = cap;
+    return FF_OK;
+}
+
 // After a counted Barnes-Hut evaluation: scans the per-particle interaction
 // counts into entry slots and sizes every buffer the recorded entries need.
+// shared: the walk wrote records (no slots for merging lists are needed).
 ff_status prepare_entries(ff_ctx* c, int64_t* ne_out, int64_t* ncells_out, int64_t* max_items_out,
-                          int64_t* pool_used)
+                          int64_t* pool_used, bool shared = false)
 {
     const int64_t n = c->n;
     cudaStream_t s = c->stream;
@@ -824,7 +886,7 @@ ff_status prepare_entries(ff_ctx* c, int64_t* ne_out, int64_t* ncells_out, int64
     int ncells_h = 0;
     FF_CUDA(c, cudaMemsetAsync(c->e_total, 0, sizeof(unsigned long long), s));
     ffk::grad_entry_counts(c->counts, n, c->e_cnt, c->e_total, s);
-    ffk::scan_exclusive(c->e_cnt, c->e_base, n, c->scan_tmp, s);
+    if (!shared) ffk::scan_exclusive(c->e_cnt, c->e_base, n, c->scan_tmp, s);
     FF_LAUNCHED(c);
     unsigned long long total = 0;
     FF_CUDA(c, cudaMemcpyAsync(&total, c->e_total, sizeof(total), cudaMemcpyDeviceToHost, s));
@@ -832,20 +894,14 @@ ff_status prepare_entries(ff_ctx* c, int64_t* ne_out, int64_t* ncells_out, int64
     unsigned taken = 0;
     FF_CUDA(c, cudaMemcpyAsync(&taken, c->p_next, sizeof(taken), cudaMemcpyDeviceToHost, s));
     if ((st = sync_and_check(c)) != FF_OK) return st;
-    *pool_used = n + (int64_t)taken;
+    *pool_used = (shared ? (n + 31) / 32 : n) + (int64_t)taken;
     // entry positions are 32-bit, with room for the recording walk's 16-byte groups
     if (total >= 0xfffffff0ull)
         return fail(c, FF_EINVAL, "too many interactions (%llu) for one gradient pass", total);
     const int64_t ne = (int64_t)total;
     const int64_t ncells = ncells_h;
     const int64_t nsrc = ncells + n;
-    if (ne > c->e_cap) {
-        const int64_t cap = ne + ne / 8 + 1024;
-        if ((st = grow(c, &c->rs_key, cap)) != FF_OK) return st;
-        if ((st = grow(c, &c->rs_mask, cap)) != FF_OK) return st;
-        if ((st = grow(c, &c->e_tmp, ffk::radix_tmp_words(cap))) != FF_OK) return st;
-        c->e_cap = cap;
-    }
+    if (!shared && (st = grow_slots(c, ne)) != FF_OK) return st;
     if (nsrc > c->s_cap) {
         const int64_t cap = nsrc + nsrc / 8 + 1024;
         if ((st = grow(c, &c->s_beg, cap)) != FF_OK) return st;
@@ -887,23 +943,25 @@ ff_status grow_pool(ff_ctx* c, int64_t chunks)
     return FF_OK;
 }
 
-ffk::EntryPool pool_of(ff_ctx* c)
+ffk::EntryPool pool_of(ff_ctx* c, bool shared = false)
 {
     ffk::EntryPool p;
     p.keys = c->p_keys;
     p.link = c->p_link;
     p.next = c->p_next;
     p.cap = (uint32_t)c->p_cap;
-    p.first = (uint32_t)c->n;
+    p.first = (uint32_t)(shared ? (c->n + 31) / 32 : c->n);
     return p;
 }
 
-// The pool ready for a recording walk: room for at least n + 1024 chunks (9 per
-// particle at first), its counter cleared.
-ff_status pool_prepare(ff_ctx* c)
+// The pool ready for a recording walk, its counter cleared: for lists 9 chunks per
+// particle at first, for records (about 30 chunks a task) 3 per 2 particles.
+ff_status pool_prepare(ff_ctx* c, bool shared = false)
 {
     ff_status st;
-    if (c->p_cap < c->n + 1024 && (st = grow_pool(c, 9 * c->n + 1024)) != FF_OK) return st;
+    const int64_t first = shared ? c->n + c->n / 2 + 1024 : 9 * c->n + 1024;
+    const int64_t least = shared ? c->n / 2 + 1024 : 2 * c->n + 1024;
+    if (c->p_cap < least && (st = grow_pool(c, first)) != FF_OK) return st;
     FF_CUDA(c, cudaMemsetAsync(c->p_next, 0, sizeof(unsigned), c->stream));
     return FF_OK;
 }
@@ -912,39 +970,43 @@ ff_status pool_prepare(ff_ctx* c)
 // a pool that ran out is grown to what the walk took and the walk redone (the
 // same field, force, counts and lists).
 template <typename R>
-ff_status pool_settle(ff_ctx* c, double theta, int include_sr, int64_t used)
+ff_status pool_settle(ff_ctx* c, double theta, int include_sr, int64_t used, bool shared)
 {
     if (used <= c->p_cap) return FF_OK;
     ff_status st;
     if ((st = grow_pool(c, used + used / 8 + 1024)) != FF_OK) return st;
     FF_CUDA(c, cudaMemsetAsync(c->p_next, 0, sizeof(unsigned), c->stream));
-    Buffers& a = c->st[c->cur];
-    ffk::bh_field_record<R>(V<R>(a.pos), V<R>(a.u), c->n, tree_of<R>(c),
-                            field_params<R>(c, theta, include_sr), V<R>(c->h), V<R>(c->f),
-                            static_cast<R*>(c->esr), c->counts, c->dflags, c->work, c->off,
-                            segs_of(c), pool_of(c), c->stream);
+    record_walk<R>(c, theta, include_sr, pool_of(c, shared));
     FF_LAUNCHED(c);
     return FF_OK;
+}
+
+// Per-task record counts of the gradient pass.
+ff_status grow_tasks(ff_ctx* c)
+{
+    if (c->t_cnt && c->t_off) return FF_OK;
+    const int64_t ntask = (c->n + 31) / 32;
+    ff_status st;
+    if ((st = grow(c, &c->t_cnt, ntask)) != FF_OK) return st;
+    return grow(c, &c->t_off, ntask + 1);
 }
 
 // After the recording walk and prepare_entries: each task's sources gathered into
 // records, packed, sorted by their place in the depth-first order and scanned
 // into entry offsets (k_grad.cu).  Waits to read the number of records.
 template <typename R>
-ff_status record_sources(ff_ctx* c, int64_t ncells, int64_t* nrec_out)
+ff_status record_sources(ff_ctx* c, int64_t ncells, int64_t* nrec_out, bool shared = false)
 {
     const int64_t n = c->n;
     const int64_t nsrc = ncells + n;
     const int64_t ntask = (n + 31) / 32;
     cudaStream_t s = c->stream;
     ff_status st;
-    if (!c->t_cnt) {
-        if ((st = grow(c, &c->t_cnt, ntask)) != FF_OK) return st;
-        if ((st = grow(c, &c->t_off, ntask + 1)) != FF_OK) return st;
-    }
+    if ((st = grow_tasks(c)) != FF_OK) return st;
     // the records of task T go to the slots of its particles (rs_key, rs_mask)
-    ffk::grad_merge_records(c->e_cnt, n, pool_of(c), c->e_base, c->rs_key, c->rs_mask,
-                            c->t_cnt, c->dflags, s);
+    if (!shared)
+        ffk::grad_merge_records(c->e_cnt, n, pool_of(c), c->e_base, c->rs_key, c->rs_mask,
+                                c->t_cnt, c->dflags, s);
     ffk::scan_exclusive(c->t_cnt, c->t_off, ntask, c->scan_tmp, s);
     ffk::grad_source_map<R>(tree_of<R>(c), ncells, c->s_src, s);
     FF_LAUNCHED(c);
@@ -962,8 +1024,14 @@ ff_status record_sources(ff_ctx* c, int64_t ncells, int64_t* nrec_out)
         if ((st = grow(c, &c->r_scan, ffk::record_scan_words(cap))) != FF_OK) return st;
         c->r_cap = cap;
     }
-    ffk::grad_pack_records(c->t_cnt, c->t_off, ntask, c->e_base, c->rs_key, c->rs_mask,
-                           c->r_key, c->r_idx, c->r_rec, s);
+    if (shared) {
+        if ((st = grow_slots(c, nrec)) != FF_OK) return st;
+        ffk::grad_pack_chunks(c->t_cnt, c->t_off, ntask, pool_of(c, true), c->r_key, c->r_idx,
+                              c->r_rec, s);
+    } else {
+        ffk::grad_pack_records(c->t_cnt, c->t_off, ntask, c->e_base, c->rs_key, c->rs_mask,
+                               c->r_key, c->r_idx, c->r_rec, s);
+    }
     int passes = 1;
     while (passes < 4 && ((uint64_t)nsrc >> (8 * passes)) != 0) ++passes;
     // the records, in task order, sorted stably by source (rs_key, rs_mask
@@ -981,6 +1049,19 @@ ff_status record_sources(ff_ctx* c, int64_t ncells, int64_t* nrec_out)
 
 // Energy -1/2 sum u.h (FP64) and its gradient with the opening decisions of
 // this evaluation frozen (k_grad.cu), in sorted order in g_pos, g_u.
+void drop_graphs(ff_ctx* c);
+
+// The children's table, which a context too large for the shared walk otherwise
+// does without, for the gradient's recording walk (the captured steps then build it).
+ff_status want_child(ff_ctx* c)
+{
+    if (c->child || c->fp64 || c->p.quadrupole || c->p.count_interactions) return FF_OK;
+    c->need_child = true;
+    ff_status st = grow(c, &c->child, 2 * (size_t)c->cap);
+    if (st == FF_OK) drop_graphs(c);
+    return st;
+}
+
 template <typename R>
 ff_status energy_grad(ff_ctx* c, int32_t algo, double theta, double* energy, bool grads)
 {
@@ -1001,16 +1082,19 @@ ff_status energy_grad(ff_ctx* c, int32_t algo, double theta, double* energy, boo
         FF_LAUNCHED(c);
     } else {
         // the field, the counts and every particle's sources in one walk
-        if ((st = pool_prepare(c)) != FF_OK) return st;
-        const ffk::EntryPool pool = pool_of(c);
+        if ((st = want_child(c)) != FF_OK) return st;
+        const bool shared = shared_records(c);
+        if ((st = grow_tasks(c)) != FF_OK) return st;
+        if ((st = pool_prepare(c, shared)) != FF_OK) return st;
+        const ffk::EntryPool pool = pool_of(c, shared);
         if ((st = eval_bh<R>(c, theta, 0, true, &pool)) != FF_OK) return st;
         int64_t ne = 0, ncells = 0, max_items = 0, used = 0;
-        if ((st = prepare_entries(c, &ne, &ncells, &max_items, &used)) != FF_OK) return st;
-        if ((st = pool_settle<R>(c, theta, 0, used)) != FF_OK) return st;
+        if ((st = prepare_entries(c, &ne, &ncells, &max_items, &used, shared)) != FF_OK) return st;
+        if ((st = pool_settle<R>(c, theta, 0, used, shared)) != FF_OK) return st;
         Buffers& a = c->st[c->cur];
         ffk::Tree<R> t = tree_of<R>(c);
         int64_t nrec = 0;
-        if ((st = record_sources<R>(c, ncells, &nrec)) != FF_OK) return st;
+        if ((st = record_sources<R>(c, ncells, &nrec, shared)) != FF_OK) return st;
         ffk::grad_source_sums_rec<R>(V<R>(a.pos), V<R>(a.u), t, ncells, n, c->r_srec, c->r_E,
                                      nrec, c->s_rbeg, c->s_beg, c->s_end, c->s_items,
                                      c->s_item_off, c->s_scan, c->i_part, max_items, c->s_G,
@@ -1245,6 +1329,7 @@ ff_status mz_sensitivity(ff_ctx* c, int64_t nsteps, int64_t every, double* mz_ou
                 if ((st = vjp_walk()) != FF_OK) return st;
             }
             c->counts_valid = false;  // entries per particle, not the counting walk's split
+            c->counts_lazy = false;
             int64_t nrec = 0;
             if ((st = record_sources<R>(c, ncells, &nrec)) != FF_OK) return st;
             ffk::vjp_source_sums_rec<R>(V<R>(a.pos), V<R>(a.u), V<R>(abar), V<R>(bbar),
@@ -1393,6 +1478,7 @@ ff_status ff_set_particles(ff_ctx* c, const void* pos, const void* u, const void
     c->have_particles = true;
     c->tree_valid = false;
     c->counts_valid = false;
+    c->counts_lazy = false;
     return FF_OK;
 }
 
@@ -1525,6 +1611,7 @@ ff_status run_steps(ff_ctx* c, int64_t nsteps)
         if (c->nsys > 0) c->sys_steps += 1;
         c->tree_valid = c->tree_valid || c->p.algo == FF_ALGO_BH;
         c->counts_valid = c->p.algo == FF_ALGO_BH && c->p.count_interactions != 0;
+        c->counts_lazy = false;
     }
     return FF_OK;
 }
@@ -1612,6 +1699,7 @@ ff_status ff_tree_info(ff_ctx* c, ff_tree_info_t* out)
     if (s != FF_OK) return s;
     if (!out) return fail(c, FF_EINVAL, "out is NULL");
     if (!c->tree_valid) return fail(c, FF_ESTATE, "no Barnes-Hut tree has been built");
+    if (c->counts_lazy) count_again<float>(c);
     if ((s = retrying(c, [&] { return sync_and_check(c); })) != FF_OK) return s;
     std::memset(out, 0, sizeof(*out));
     uint32_t nc = 0;
@@ -1725,6 +1813,7 @@ ff_status ff_get_counts(ff_ctx* c, int32_t* accepted, int32_t* pairs, int32_t* o
     LaunchTally tally_(c);
     ff_status s = usable(c, true);
     if (s != FF_OK) return s;
+    if (c->counts_lazy) count_again<float>(c);
     if (!c->counts_valid) return fail(c, FF_ESTATE, "no interaction counts recorded (count_interactions = 0 or no BH evaluation)");
     const int64_t n = c->n;
     int32_t* stg = static_cast<int32_t*>(c->staging);
@@ -1804,6 +1893,7 @@ ff_status ff_set_systems(ff_ctx* c, int32_t nsys, const int64_t* counts, const d
     c->sys_steps = 0;
     c->tree_valid = false;
     c->counts_valid = false;
+    c->counts_lazy = false;
     return FF_OK;
 }
 

@@ -287,6 +287,9 @@ void grad_source_map(Tree<R> t, int64_t ncells, uint32_t* src_of, cudaStream_t s
 void grad_pack_records(const uint32_t* tcount, const uint32_t* toff, int64_t ntask,
                        const uint32_t* base, const uint32_t* rkeys, const uint32_t* rmask,
                        uint32_t* ckey, uint32_t* cidx, uint2* crec, cudaStream_t s);
+// The same from the chunks of warp_walk_record.
+void grad_pack_chunks(const uint32_t* tcount, const uint32_t* toff, int64_t ntask, EntryPool pool,
+                      uint32_t* ckey, uint32_t* cidx, uint2* crec, cudaStream_t s);
 // After the records are sorted by key (skey, sidx = their packed index):
 // srec[i] = crec[sidx[i]], recE[i] = entries before record i (recE[nrec] =
 // entries), and per source s = src_of[key] its first record rbeg, and the
@@ -392,6 +395,16 @@ constexpr int64_t kWarpWalkCells = int64_t(1) << 29;
 void warp_walk(const float4* pos, const float4* u, int64_t n, Tree<float> t,
                FieldParams<float> fp, float4* h, float4* f, float* esr, int* flags, int* work,
                const uint32_t* off, Segs sg, cudaStream_t s);
+
+// The same walk for the gradient pass (any n), tasks of 32: also each task's
+// records (source key, lanes that have it), in no particular order, to chunks of
+// kPoolChunk / 2 in the pool (task T's first chunk is T, pool.first = the number of
+// tasks), their number to tcount[T], and each particle's number of sources to
+// counts[k].x.
+void warp_walk_record(const float4* pos, const float4* u, int64_t n, Tree<float> t,
+                      FieldParams<float> fp, float4* h, float4* f, float* esr, int4* counts,
+                      uint32_t* tcount, int* flags, int* work, const uint32_t* off, Segs sg,
+                      EntryPool pool, cudaStream_t s);
 
 // The FP64 walk without dipole-position terms, with or without counts
 // (k_walk64.cu).  Needs t.child; t.cap <= kWarpWalkCells.

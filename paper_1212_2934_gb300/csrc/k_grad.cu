@@ -266,6 +266,36 @@ __global__ void k_pack_records(const uint32_t* __restrict__ tcount,
     }
 }
 
+// One warp per task: its records from the chunks of the recording walk, packed in
+// task order, two records a lane, the next chunk's link read with them.
+__global__ void k_pack_chunks(const uint32_t* __restrict__ tcount,
+                              const uint32_t* __restrict__ toff, int64_t ntask, EntryPool pool,
+                              uint32_t* __restrict__ ckey, uint32_t* __restrict__ cidx,
+                              uint2* __restrict__ crec)
+{
+    constexpr uint32_t kChunk = kPoolChunk / 2;
+    const int64_t task = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint32_t lane = threadIdx.x & 31;
+    if (task >= ntask) return;
+    const uint32_t cnt = tcount[task], dst = toff[task];
+    const uint2* rec = reinterpret_cast<const uint2*>(pool.keys);
+    uint32_t ck = (uint32_t)task;
+    for (uint32_t r0 = 0; r0 < cnt && ck < pool.cap; r0 += kChunk) {
+        const uint32_t next = r0 + kChunk < cnt ? pool.link[ck] : ck;
+#pragma unroll
+        for (uint32_t q = 0; q < kChunk; q += 32) {
+            const uint32_t r = r0 + q + lane;
+            if (r < cnt) {
+                const uint2 v = rec[(size_t)ck * kChunk + q + lane];
+                ckey[dst + r] = v.x;
+                cidx[dst + r] = dst + r;
+                crec[dst + r] = make_uint2((uint32_t)task, v.y);
+            }
+        }
+        ck = next;
+    }
+}
+
 // The sorted records in one pass: srec[i] = crec[sidx[i]], recE[i] = the
 // entries (set mask bits) of the records before i, and per source s = src_of[key]
 // its first record rbeg[s] and entry range [beg[s], end[s]) (keys outside
@@ -767,6 +797,15 @@ void grad_pack_records(const uint32_t* tcount, const uint32_t* toff, int64_t nta
     const int64_t g = ntask < (1 << 20) ? ntask : (1 << 20);
     k_pack_records<<<(unsigned)g, kGradThreads, 0, s>>>(tcount, toff, ntask, base, rkeys, rmask,
                                                         ckey, cidx, crec);
+    counted();
+}
+
+void grad_pack_chunks(const uint32_t* tcount, const uint32_t* toff, int64_t ntask, EntryPool pool,
+                      uint32_t* ckey, uint32_t* cidx, uint2* crec, cudaStream_t s)
+{
+    if (ntask <= 0) return;
+    k_pack_chunks<<<blocks(ntask * 32, kGradThreads), kGradThreads, 0, s>>>(tcount, toff, ntask, pool,
+                                                                           ckey, cidx, crec);
     counted();
 }
 

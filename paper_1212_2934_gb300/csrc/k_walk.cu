@@ -62,6 +62,42 @@ struct Sums {
     float hx, hy, hz, fx, fy, fz, sx, sy, sz, es;
 };
 
+// The records of a task (energy gradient): each source once, with the lanes that
+// have it, 64 to a chunk of the pool (the task's own chunk first, then chunks
+// handed out by a counter, linked; chunks at or past cap are not written).
+constexpr uint32_t kRecChunk = kPoolChunk / 2;
+
+struct RecordWriter {
+    uint32_t ck, fill, total;
+    int nsrc;  // this lane's sources
+
+    __device__ __forceinline__ void put(const EntryPool& p, bool valid, uint32_t key, uint32_t mask)
+    {
+        const int lane = threadIdx.x & 31;
+        const uint32_t m = __ballot_sync(kFull, valid), c = (uint32_t)__popc(m);
+        const uint32_t at = fill + (uint32_t)__popc(m & ((1u << lane) - 1u));
+        const bool full = fill + c >= kRecChunk;  // the chunk after a full one is taken at once
+        uint32_t nk = 0;
+        if (full) {
+            if (lane == 0) {
+                nk = p.first + atomicAdd(p.next, 1u);
+                if (ck < p.cap) p.link[ck] = nk;
+            }
+            nk = __shfl_sync(kFull, nk, 0);
+        }
+        const uint32_t to = at < kRecChunk ? ck : nk;
+        if (valid && to < p.cap)
+            reinterpret_cast<uint2*>(p.keys)[(size_t)to * kRecChunk + at % kRecChunk] =
+                make_uint2(key, mask);
+        fill += c;
+        total += c;
+        if (full) {
+            ck = nk;
+            fill -= kRecChunk;
+        }
+    }
+};
+
 // What one source adds for this lane beyond the dipole terms of an ordinary
 // separation (rare): the LJ force of a particle within the cut, where a
 // one-particle leaf is first decided between accepting it and summing it as a
@@ -122,11 +158,14 @@ __device__ __forceinline__ void add_if(uint32_t mask, uint32_t bit, float r2, fl
           "f"(sx), "f"(sy), "f"(sz), "r"(one));
 }
 
-// Sums the first cnt sources of the list.
+// Sums the first cnt sources of the list (REC: and records the cells among them;
+// particles are recorded where their leaf is opened).
+template <bool REC>
 __device__ __forceinline__ void sum_sources(WarpShared& w, int cnt, const Tree<float>& t,
                                             const FieldParams<float>& fp, float near2,
                                             const float4* __restrict__ pos,
-                                            const float4* __restrict__ u, const Target& k, Sums& a)
+                                            const float4* __restrict__ u, const Target& k, Sums& a,
+                                            RecordWriter& rw, const EntryPool& ep)
 {
     const int lane = threadIdx.x & 31;
     const uint32_t bit = 1u << lane;
@@ -143,6 +182,13 @@ __device__ __forceinline__ void sum_sources(WarpShared& w, int cnt, const Tree<f
                 const bool p = (e.x & kParticle) != 0u;
                 c = p ? pos[i] : t.cell[i].cen;
                 m = p ? u[i] : t.mom[i];
+            }
+            if (REC) {
+                const uint32_t i = e.x & kIndex;
+                const bool cell = b + lane < cnt && !(e.x & kParticle);
+                // named by its place in the depth-first order of cells and particles
+                const uint32_t key = cell ? i + (uint32_t)t.cell[i].node.x : 0u;
+                rw.put(ep, cell, key, e.y);
             }
             float* st = w.stage + (lane >> 1) * kPairWords + (lane & 1);
             st[0] = -c.x;
@@ -167,6 +213,7 @@ __device__ __forceinline__ void sum_sources(WarpShared& w, int cnt, const Tree<f
             const float2 ry = __fadd2_rn(ky, make_float2(q0.z, q0.w));
             const float2 rz = __fadd2_rn(kz, make_float2(q1.x, q1.y));
             const float2 r2 = pair_r2_2(rx, ry, rz);
+            if (REC) rw.nsrc += ((mk.x & bit) != 0u ? 1 : 0) + ((mk.y & bit) != 0u ? 1 : 0);
             const float2 ir = make_float2(rsqrt_normal(r2.x), rsqrt_normal(r2.y));
             const DipoleTerms2 d =
                 dipole2(rx, ry, rz, ir, ukx, uky, ukz, make_float2(q1.z, q1.w),
@@ -193,13 +240,15 @@ __device__ __forceinline__ void sum_sources(WarpShared& w, int cnt, const Tree<f
 
 // Sums the list's full batches of 32 and moves the rest to its front; returns
 // how many that is.
+template <bool REC>
 __device__ __forceinline__ int sum_full(WarpShared& w, int cnt, const Tree<float>& t,
                                         const FieldParams<float>& fp, float near2,
                                         const float4* __restrict__ pos,
-                                        const float4* __restrict__ u, const Target& k, Sums& a)
+                                        const float4* __restrict__ u, const Target& k, Sums& a,
+                                        RecordWriter& rw, const EntryPool& ep)
 {
     const int lane = threadIdx.x & 31, full = cnt & ~31;
-    sum_sources(w, full, t, fp, near2, pos, u, k, a);
+    sum_sources<REC>(w, full, t, fp, near2, pos, u, k, a, rw, ep);
     uint2 e = make_uint2(0u, 0u);
     if (lane < cnt - full) e = w.q.list[full + lane];
     __syncwarp();
@@ -215,14 +264,15 @@ __device__ __forceinline__ float warp_min(float v)
     return v;
 }
 
-template <int T>
+template <int T, bool REC>
 __device__ __forceinline__ void walk_task(WarpShared& w, int task, const float4* __restrict__ pos,
                                           const float4* __restrict__ u, int n,
                                           const Tree<float>& t, const FieldParams<float>& fp,
                                           unsigned ncells, float4* __restrict__ h,
                                           float4* __restrict__ f, float* __restrict__ esr,
                                           int* flags, const uint32_t* __restrict__ off,
-                                          const Segs& sg)
+                                          const Segs& sg, const EntryPool& ep,
+                                          int4* __restrict__ counts, uint32_t* __restrict__ tcount)
 {
     const int lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
@@ -256,6 +306,7 @@ __device__ __forceinline__ void walk_task(WarpShared& w, int task, const float4*
             if (lead) w.q.stack[top - 1 - __popc(lm & lt)] = make_uint2(off[sg.start[sys]], mine);
         }
     }
+    RecordWriter rw = {(uint32_t)task, 0u, 0u, 0};
     int cnt = 0;
     unsigned rounds = 0;
     while (top > 0) {
@@ -274,9 +325,10 @@ __device__ __forceinline__ void walk_task(WarpShared& w, int task, const float4*
                 uint32_t mask = s < nd.y ? first.y : 0u;
                 if (s >= k0 && s < k0 + T) mask &= ~(1u << (s - k0));
                 const uint32_t keep = __ballot_sync(kFull, mask != 0u);
+                if (REC) rw.put(ep, mask != 0u, (first.x & kIndex) + 1u + (uint32_t)s, mask);
                 if (mask) w.q.list[cnt + __popc(keep & lt)] = make_uint2((uint32_t)s | kParticle, mask);
                 cnt += __popc(keep);
-                if (cnt >= kBatch) cnt = sum_full(w, cnt, t, fp, near2, pos, u, tg, a);
+                if (cnt >= kBatch) cnt = sum_full<REC>(w, cnt, t, fp, near2, pos, u, tg, a, rw, ep);
             }
             --top;
             continue;
@@ -367,7 +419,7 @@ __device__ __forceinline__ void walk_task(WarpShared& w, int task, const float4*
         cnt += emit;
         if (cnt >= kBatch) {
             __syncwarp();
-            cnt = sum_full(w, cnt, t, fp, near2, pos, u, tg, a);
+            cnt = sum_full<REC>(w, cnt, t, fp, near2, pos, u, tg, a, rw, ep);
         }
         // every round opens a cell or clears its part of the stack
         if (++rounds > max_rounds) {  // a damaged tree
@@ -376,8 +428,10 @@ __device__ __forceinline__ void walk_task(WarpShared& w, int task, const float4*
         }
     }
     __syncwarp();
-    sum_sources(w, cnt, t, fp, near2, pos, u, tg, a);
+    sum_sources<REC>(w, cnt, t, fp, near2, pos, u, tg, a, rw, ep);
+    if (REC && lane == 0) tcount[task] = rw.total;
     if (!active) return;
+    if (REC) counts[k] = make_int4(rw.nsrc, 0, 0, 0);
     float4 ho, fo;
     ho.x = fp.dip_scale * a.hx;
     ho.y = fp.dip_scale * a.hy;
@@ -392,12 +446,13 @@ __device__ __forceinline__ void walk_task(WarpShared& w, int task, const float4*
     if (esr) esr[k] = a.es;
 }
 
-template <int T>
+template <int T, bool REC>
 __global__ void __launch_bounds__(kWalkThreads, kWalkBlocks) k_warp_walk(
     const float4* __restrict__ pos, const float4* __restrict__ u, int n, Tree<float> t,
     FieldParams<float> fp, float4* __restrict__ h, float4* __restrict__ f,
     float* __restrict__ esr, int* flags, int* __restrict__ work, int nseg,
-    const uint32_t* __restrict__ off, Segs sg)
+    const uint32_t* __restrict__ off, Segs sg, EntryPool ep, int4* __restrict__ counts,
+    uint32_t* __restrict__ tcount)
 {
     extern __shared__ __align__(16) unsigned char walk_smem[];
     WarpShared& w = reinterpret_cast<WarpShared*>(walk_smem)[threadIdx.x >> 5];
@@ -419,20 +474,23 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkBlocks) k_warp_walk(
             got = __shfl_sync(kFull, got, 0);
             const int task = t0 + got;
             if (task >= t1) break;
-            walk_task<T>(w, task, pos, u, n, t, fp, ncells, h, f, esr, flags, off, sg);
+            walk_task<T, REC>(w, task, pos, u, n, t, fp, ncells, h, f, esr, flags, off, sg, ep,
+                              counts, tcount);
         }
     }
 }
 
-template <int T>
+template <int T, bool REC = false>
 void warp_walk_launch(const float4* pos, const float4* u, int64_t n, Tree<float> t,
                       FieldParams<float> fp, float4* h, float4* f, float* esr, int* flags,
-                      int* work, const uint32_t* off, Segs sg, cudaStream_t s)
+                      int* work, const uint32_t* off, Segs sg, cudaStream_t s,
+                      const EntryPool& ep = EntryPool(), int4* counts = nullptr,
+                      uint32_t* tcount = nullptr)
 {
     constexpr int smem = (int)sizeof(WarpShared) * (kWalkThreads / 32);
     static std::mutex mu;
     static PersistentGrid cache[kMaxDevices];
-    const auto kern = k_warp_walk<T>;
+    const auto kern = k_warp_walk<T, REC>;
     const PersistentGrid g = persistent_grid(cache, mu, [kern] {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -443,7 +501,7 @@ void warp_walk_launch(const float4* pos, const float4* u, int64_t n, Tree<float>
     });
     cudaMemsetAsync(work, 0, sizeof(int) * g.nseg, s);
     kern<<<g.blocks, kWalkThreads, smem, s>>>(pos, u, (int)n, t, fp, h, f, esr, flags, work, g.nseg,
-                                         off, sg);
+                                              off, sg, ep, counts, tcount);
 }
 
 }  // namespace
@@ -464,6 +522,21 @@ void warp_walk(const float4* pos, const float4* u, int64_t n, Tree<float> t,
         warp_walk_launch<16>(pos, u, n, t, fp, h, f, esr, flags, work, off, sg, s);
     else
         warp_walk_launch<32>(pos, u, n, t, fp, h, f, esr, flags, work, off, sg, s);
+}
+
+// The walk of the gradient pass, at any n: lists gathered from the one-lane walk
+// (its counting instance writing every particle's sources, and a hash table per
+// task merging 32 lists) cost 1.1 ms of 5.2 at n = 262,144.  Here a task's sources
+// are known once, with the lanes that have them, as the walk goes.
+void warp_walk_record(const float4* pos, const float4* u, int64_t n, Tree<float> t,
+                      FieldParams<float> fp, float4* h, float4* f, float* esr, int4* counts,
+                      uint32_t* tcount, int* flags, int* work, const uint32_t* off, Segs sg,
+                      EntryPool pool, cudaStream_t s)
+{
+    if (n <= 0) return;
+    warp_walk_launch<32, true>(pos, u, n, t, fp, h, f, esr, flags, work, off, sg, s, pool, counts,
+                               tcount);
+    counted();
 }
 
 }  // namespace ffk

@@ -134,3 +134,26 @@ def test_fp64_tasks_spanning_systems(ff):
         h, f = ff.ff_dipolar_field(ctx, ff.FF_ALGO_BH, 0.5, True)
         assert np.array_equal(h, hp[off:off + k]) and np.array_equal(f, fp[off:off + k])
         off += k
+
+
+@pytest.mark.parametrize("leaf_max", [1, 6])
+@pytest.mark.parametrize("n", [1, 31, 33, 3001, 120011])
+def test_gradient_records_match_lists(ff, n, leaf_max):
+    """The gradient from the shared walk's records and from the lists of the counting walk (a
+    context that counts): the same sources in the same order, so the same bits; and the counts
+    of the gradient's evaluation can be asked for after either."""
+    pos, u = _gas(n, n + leaf_max)
+    if n > 3000:
+        pos[11:60] = pos[11]  # a leaf of several particles at any leaf_max
+    res = []
+    for count in (0, 1):
+        ctx = ff.ff_create(ff.ff_params_default(n=n, leaf_max=leaf_max, count_interactions=count))
+        ff.ff_set_particles(ctx, pos, u)
+        e, gp, gu = ff.ff_energy_grad(ctx, ff.FF_ALGO_BH, 0.5, dtype=np.float32)
+        e2, gp2, gu2 = ff.ff_energy_grad(ctx, ff.FF_ALGO_BH, 0.5, dtype=np.float32)
+        assert e == e2 and np.array_equal(gp, gp2) and np.array_equal(gu, gu2)
+        res.append((e, gp, gu, *ff.ff_get_counts(ctx), ff.ff_tree_info(ctx)["interactions"]))
+        ff.ff_step(ctx, 2)  # steps after a gradient
+        res[-1] += tuple(ff.ff_get_particles(ctx))
+    for a, b in zip(*res):
+        assert np.array_equal(a, b)
