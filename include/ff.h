@@ -393,7 +393,7 @@ const char *ff_status_string(ff_status s);
  *
  * Nothing is allocated: besides the caller's buffers the work uses one fixed
  * scratch array inside the library, sized for n <= FF_NOALLOC_MAX_N (about
- * 3.7 MB, held on every GPU that loads the library until the process exits).
+ * 3.9 MB, held on every GPU that loads the library until the process exits).
  * The first call on a device looks up the array's device address and keeps
  * it for the life of the process: make that first call before any stream
  * capture on that device, and do not use the call on a device after

@@ -11,7 +11,7 @@
 // cannot be issued while that stream is being captured into a graph.
 //
 // The scratch array is a static device variable: every GPU that loads the
-// library keeps it (about 3.7 MB) until the process exits.  Its name in host
+// library keeps it (about 3.9 MB) until the process exits.  Its name in host
 // code is only a host-side stand-in, so the device address is looked up with
 // cudaGetSymbolAddress, once per device, on the first call made with that
 // device current; the address is kept for the life of the process, so the

@@ -46,28 +46,42 @@ constexpr int kRadixBins = 1 << kRadixBits;
 // digit (alternate passes use alternate arrays; each tile clears its words in
 // the other array for the pass after it), then one tile ticket per pass.
 constexpr int kOsThreads = 256;  // = kRadixBins: one digit per thread
-constexpr int kOsItems = 16;     // keys per thread per tile
-constexpr int kOsTile = kOsThreads * kOsItems;  // the smallest tile (sizes the scratch)
-// Large tiles carry many bytes per look-back and per block-wide scan, and
-// keep the look-back chains of a pass short (all tiles of a 1M-key pass run
-// at once).  The tile is staged in dynamic shared memory.
-// 32-bit keys (the gradient's entries, hundreds of millions) take twice as
-// many per thread: 8192-key tiles in the same shared memory.
+// Keys per thread of a tile.  Large tiles carry many bytes per look-back and per
+// block-wide scan and keep the look-back chains of a pass short (all tiles of a
+// 1M-key pass run at once): 16 for 64-bit keys, 32 for 32-bit ones (the gradient's
+// records, tens of millions), in the same shared memory.  With few keys a pass
+// lasts as long as one tile, so tiles are smaller: us a sort of 64-bit keys with
+// 16 / 8 / 4 keys a thread: n = 50,021 115 / 99 / 84; 100,003 116 / 100 / 100;
+// 262,144 140 / 124 / 128; 1,048,576 197 / 210 / 268.
 template <typename K>
-constexpr int os_items() { return sizeof(K) == 4 ? 2 * kOsItems : kOsItems; }
-template <typename K>
-constexpr int os_min_blocks() { return 2; }
-template <typename K>
+constexpr int os_items(int64_t n)
+{
+    return sizeof(K) == 4 ? (n <= 262144 ? 8 : 32) : n <= 65536 ? 4 : n <= 393216 ? 8 : 16;
+}
+constexpr int64_t kOsTile = kOsThreads * 16;  // the largest tile of 64-bit keys
+template <typename K, int ITEMS>
 constexpr size_t os_dyn_smem()
 {
-    return (size_t)kOsThreads * os_items<K>() * (sizeof(K) + sizeof(uint32_t));
+    return (size_t)kOsThreads * ITEMS * (sizeof(K) + sizeof(uint32_t));
 }
 constexpr int kOsMaxPasses = 8;
-constexpr int64_t os_tiles(int64_t n) { return (n + kOsTile - 1) / kOsTile; }
+template <typename K>
+constexpr int64_t os_tiles(int64_t n)
+{
+    return (n + kOsThreads * os_items<K>(n) - 1) / (kOsThreads * os_items<K>(n));
+}
+// Words of scratch for up to n keys of either kind (fewer keys in smaller tiles
+// may have more tiles than n).
 constexpr size_t os_tmp_words(int64_t n)
 {
-    return (size_t)kOsMaxPasses * kRadixBins + 4 * (size_t)kRadixBins * (size_t)os_tiles(n) +
-           kOsMaxPasses;
+    int64_t tiles = os_tiles<uint64_t>(n);
+    const int64_t edges[] = {65536, 393216};
+    for (int64_t e : edges)
+        if (e < n && os_tiles<uint64_t>(e) > tiles) tiles = os_tiles<uint64_t>(e);
+    const int64_t small = n < 262144 ? n : 262144;
+    if (os_tiles<uint32_t>(small) > tiles) tiles = os_tiles<uint32_t>(small);
+    if (os_tiles<uint32_t>(n) > tiles) tiles = os_tiles<uint32_t>(n);
+    return (size_t)kOsMaxPasses * kRadixBins + 4 * (size_t)kRadixBins * (size_t)tiles + kOsMaxPasses;
 }
 
 // Root cube, written by the bbox kernels and read by the key kernel.

@@ -8,6 +8,7 @@
 // running), each bounded, so every loop ends.
 #include <climits>
 #include <mutex>
+#include <type_traits>
 
 #include "ffk.cuh"
 
@@ -177,19 +178,19 @@ constexpr int kOsWindow = 8;                             // status words read pe
 // bounded.  The tile is reordered in shared memory by digit before the look-back
 // and written after it, consecutive threads storing consecutive elements of
 // one run.
-template <typename K>
-__global__ void __launch_bounds__(kOsThreads, os_min_blocks<K>()) k_os_scatter(
+template <typename K, int ITEMS>
+__global__ void __launch_bounds__(kOsThreads, ITEMS >= 16 ? 2 : 4) k_os_scatter(
     const K* __restrict__ kin, const uint32_t* __restrict__ vin, K* __restrict__ kout,
     uint32_t* __restrict__ vout, int64_t n, int shift, const uint32_t* __restrict__ hist,
     unsigned long long* status, unsigned long long* __restrict__ status_next,
     uint32_t* ticket, int* flags, const uint32_t* __restrict__ sysd, int withhold)
 {
     constexpr int kWarps = kOsThreads / 32;
-    constexpr int kItems = os_items<K>();
+    constexpr int kItems = ITEMS;
     constexpr int kTile = kOsThreads * kItems;
     constexpr int kWarpItems = kTile / kWarps;
     static_assert(kWarpItems == 32 * kItems, "each warp ranks kItems rounds of 32");
-    extern __shared__ __align__(16) unsigned char os_smem[];  // os_dyn_smem<K>() bytes
+    extern __shared__ __align__(16) unsigned char os_smem[];  // os_dyn_smem<K, ITEMS>() bytes
     K* s_key = reinterpret_cast<K*>(os_smem);
     uint32_t* s_val = reinterpret_cast<uint32_t*>(os_smem + sizeof(K) * kTile);
     __shared__ uint32_t s_wcnt[kWarps][kRadixBins];  // per-warp digit counts, then prefixes
@@ -1111,7 +1112,7 @@ void scan_exclusive(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* tmp,
 
 // The scatter's tile needs more dynamic shared memory than the default limit;
 // the limit is raised once per device.
-template <typename K>
+template <typename K, int ITEMS>
 void os_prepare()
 {
     static std::mutex mu;
@@ -1120,9 +1121,20 @@ void os_prepare()
     cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lock(mu);
     if (dev >= 0 && dev < 64 && done[dev]) return;
-    cudaFuncSetAttribute(k_os_scatter<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)os_dyn_smem<K>());
+    cudaFuncSetAttribute(k_os_scatter<K, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)os_dyn_smem<K, ITEMS>());
     if (dev >= 0 && dev < 64) done[dev] = true;
+}
+
+template <typename K, int ITEMS>
+void os_pass(const K* ka, const uint32_t* va, K* kb, uint32_t* vb, int64_t n, int64_t tiles,
+             int shift, const uint32_t* hist, unsigned long long* status,
+             unsigned long long* status_next, uint32_t* ticket, int* flags, const uint32_t* sysd,
+             int withhold, cudaStream_t s)
+{
+    os_prepare<K, ITEMS>();
+    k_os_scatter<K, ITEMS><<<(unsigned)tiles, kOsThreads, os_dyn_smem<K, ITEMS>(), s>>>(
+        ka, va, kb, vb, n, shift, hist, status, status_next, ticket, flags, sysd, withhold);
 }
 
 size_t radix_tmp_words(int64_t n) { return os_tmp_words(n); }
@@ -1136,7 +1148,7 @@ bool os_sort(K* k0, uint32_t* v0, K* k1, uint32_t* v1, int64_t n, uint32_t* tmp,
     if (n <= 1 || passes < 1) return false;
     if (passes > kOsMaxPasses) passes = kOsMaxPasses;
     if (!sysd && passes * kRadixBits > (int)(8 * sizeof(K))) passes = (int)(8 * sizeof(K)) / kRadixBits;
-    const int64_t tiles = (n + kOsThreads * os_items<K>() - 1) / (kOsThreads * os_items<K>());
+    const int64_t tiles = os_tiles<K>(n);
     uint32_t* hist = tmp;
     unsigned long long* status[2];
     status[0] = reinterpret_cast<unsigned long long*>(tmp + kOsMaxPasses * kRadixBins);
@@ -1154,11 +1166,18 @@ bool os_sort(K* k0, uint32_t* v0, K* k1, uint32_t* v1, int64_t n, uint32_t* tmp,
     uint32_t* va = v0;
     K* kb = k1;
     uint32_t* vb = v1;
-    os_prepare<K>();
+    constexpr int kLarge = sizeof(K) == 4 ? 32 : 16;
     for (int p = 0; p < passes; ++p) {
-        k_os_scatter<K><<<(unsigned)tiles, kOsThreads, os_dyn_smem<K>(), s>>>(
-            ka, va, kb, vb, n, p * kRadixBits, hist + p * kRadixBins, status[p & 1],
-            status[(p + 1) & 1], tickets + p, flags, sysd, withhold);
+        const auto pass = [&](auto items) {
+            os_pass<K, decltype(items)::value>(ka, va, kb, vb, n, tiles, p * kRadixBits,
+                                               hist + p * kRadixBins, status[p & 1],
+                                               status[(p + 1) & 1], tickets + p, flags, sysd,
+                                               withhold, s);
+        };
+        const int items = os_items<K>(n);
+        if (items == kLarge) pass(std::integral_constant<int, kLarge>());
+        else if (items == 8) pass(std::integral_constant<int, 8>());
+        else if constexpr (sizeof(K) == 8) pass(std::integral_constant<int, 4>());
         K* tk = ka; ka = kb; kb = tk;
         uint32_t* tv = va; va = vb; vb = tv;
     }
