@@ -509,14 +509,16 @@ void warp_walk_launch(const float4* pos, const float4* u, int64_t n, Tree<float>
 // Targets per warp: the chip holds 2432 such warps.  Fewer targets a task mean
 // more tasks in flight and fewer sources in each (a task of 8 passes 1180 cells
 // on average where one of 32 passes 1700), but more work in all.  Measured on
-// GB300, gases at volume fraction 0.05, ms per walk with 8 / 16 / 32 targets:
-//   n = 1,000  0.167 / 0.178 / 0.190     n = 16,384  0.337 / 0.316 / 0.334
-//   n = 4,096  0.218 / 0.237 / 0.257     n = 32,768  0.511 / 0.453 / 0.412
+// GB300, gases at volume fraction 0.05, ms per walk with 4 / 8 / 16 / 32 targets:
+//   n = 1,000  0.161 / 0.167 / 0.178 / 0.190     n = 16,384  - / 0.337 / 0.316 / 0.334
+//   n = 4,000  0.212 / 0.220 / 0.237 / 0.257     n = 32,768  - / 0.511 / 0.453 / 0.412
 void warp_walk(const float4* pos, const float4* u, int64_t n, Tree<float> t,
                FieldParams<float> fp, float4* h, float4* f, float* esr, int* flags, int* work,
                const uint32_t* off, Segs sg, cudaStream_t s)
 {
-    if (n <= 8192)
+    if (n <= 4096)
+        warp_walk_launch<4>(pos, u, n, t, fp, h, f, esr, flags, work, off, sg, s);
+    else if (n <= 8192)
         warp_walk_launch<8>(pos, u, n, t, fp, h, f, esr, flags, work, off, sg, s);
     else if (n <= 26624)
         warp_walk_launch<16>(pos, u, n, t, fp, h, f, esr, flags, work, off, sg, s);

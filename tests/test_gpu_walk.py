@@ -3,7 +3,7 @@
 the oracle.
 
 Contexts of up to 106,496 particles without interaction counts take a walk in which a warp
-serves 8, 16 or 32 particles (n <= 8192, <= 26,624, above); with counts they take the one-lane
+serves 4, 8, 16 or 32 particles (n <= 4096, <= 8192, <= 26,624, above); with counts they take the one-lane
 walk.  Both add every particle's sources in the same order with the same operations, so fields
 and forces agree bit for bit, over the edges of the task sizes, leaves of several particles,
 LJ on and off, opening angles from 0 (every cell opened) to 0.9, tasks that span several
@@ -47,7 +47,7 @@ def _both(ff, pos, u, theta, sizes=None, dtype=np.float32, **kw):
     return out
 
 
-@pytest.mark.parametrize("n", [1, 2, 7, 9, 33, 1000, 8191, 8193, 26623, 26625, 40009, 106496])
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 9, 33, 1000, 4095, 4097, 8191, 8193, 26623, 26625, 40009, 106496])
 def test_equals_counting_walk_at_task_edges(ff, n):
     pos, u = _gas(n, n)
     (hp, fp), (hc, fc) = _both(ff, pos, u, 0.5)
