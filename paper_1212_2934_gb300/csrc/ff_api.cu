@@ -722,38 +722,36 @@ const char* check_params(const ff_params* p)
     return nullptr;
 }
 
-template <typename R>
-ff_status load_array(ff_ctx* c, const void* src, int32_t dtype, int32_t loc, void* dst, int slot)
+template <typename R, typename I>
+void load_state(ff_ctx* c, const void* const src[4])
 {
-    const int64_t n = c->n;
-    if (!src) {
-        ffk::fill_zero4<R>(V<R>(dst), n, c->stream);
-        return FF_OK;
+    Buffers& a = c->st[c->cur];
+    ffk::In4<I> in;
+    ffk::Out4<ffk::vec4<R>> out;
+    void* dst[4] = {a.pos, a.u, a.vel, a.om};
+    for (int q = 0; q < 4; ++q) {
+        in.p[q] = static_cast<const I*>(src[q]);
+        out.p[q] = V<R>(dst[q]);
     }
-    const void* dsrc = src;
-    if (loc == FF_HOST) {
-        char* stg = static_cast<char*>(c->staging) + (size_t)slot * 3 * n * sizeof(double);
-        FF_CUDA(c, cudaMemcpyAsync(stg, src, 3 * n * dsize(dtype), cudaMemcpyHostToDevice, c->stream));
-        dsrc = stg;
-    }
-    if (dtype == FF_DTYPE_F64)
-        ffk::load3<R, double>(static_cast<const double*>(dsrc), n, V<R>(dst), c->stream);
-    else
-        ffk::load3<R, float>(static_cast<const float*>(dsrc), n, V<R>(dst), c->stream);
-    return FF_OK;
+    ffk::load_state<R, I>(in, c->n, out, a.id, c->stream);
 }
 
 template <typename R>
 ff_status set_particles(ff_ctx* c, const void* pos, const void* u, const void* vel,
                         const void* om, int32_t dtype, int32_t loc)
 {
-    Buffers& a = c->st[c->cur];
-    ff_status s;
-    if ((s = load_array<R>(c, pos, dtype, loc, a.pos, 0)) != FF_OK) return s;
-    if ((s = load_array<R>(c, u, dtype, loc, a.u, 1)) != FF_OK) return s;
-    if ((s = load_array<R>(c, vel, dtype, loc, a.vel, 2)) != FF_OK) return s;
-    if ((s = load_array<R>(c, om, dtype, loc, a.om, 3)) != FF_OK) return s;
-    ffk::iota32(a.id, c->n, c->stream);
+    const size_t bytes = 3 * (size_t)c->n * dsize(dtype);
+    const void* src[4] = {pos, u, vel, om};
+    for (int q = 0; q < 4; ++q) {
+        if (!src[q] || loc != FF_HOST) continue;
+        char* stg = static_cast<char*>(c->staging) + (size_t)q * 3 * c->n * sizeof(double);
+        FF_CUDA(c, cudaMemcpyAsync(stg, src[q], bytes, cudaMemcpyHostToDevice, c->stream));
+        src[q] = stg;
+    }
+    if (dtype == FF_DTYPE_F64)
+        load_state<R, double>(c, src);
+    else
+        load_state<R, float>(c, src);
     // a new state: earlier flags no longer apply, and steps that a too small cell array
     // held back are dropped with the state they were for (the noise counter follows
     // the host's step count)
@@ -765,26 +763,41 @@ ff_status set_particles(ff_ctx* c, const void* pos, const void* u, const void* v
     return FF_OK;
 }
 
-// Writes one record array (sorted order) to a caller array in caller order.
+// Writes up to four record arrays (sorted order) to caller arrays in caller order
+// (null: left out).
 template <typename R>
-ff_status store_array(ff_ctx* c, const void* src, const uint32_t* id, void* dst, int32_t dtype,
-                      int32_t loc, int slot)
+ff_status store_arrays(ff_ctx* c, const void* const src[4], void* const dst[4], int32_t dtype,
+                       int32_t loc)
 {
-    if (!dst) return FF_OK;
     const int64_t n = c->n;
-    void* ddst = dst;
-    char* stg = static_cast<char*>(c->staging) + (size_t)slot * 3 * n * sizeof(double);
-    if (loc == FF_HOST) ddst = stg;
-    StageTimer tm(c, S_OUT);
-    if (dtype == FF_DTYPE_F64)
-        ffk::scatter3<R, double>(static_cast<const ffk::vec4<R>*>(src), id, n,
-                                 static_cast<double*>(ddst), c->stream);
-    else
-        ffk::scatter3<R, float>(static_cast<const ffk::vec4<R>*>(src), id, n,
-                                static_cast<float*>(ddst), c->stream);
+    const uint32_t* id = c->st[c->cur].id;
+    const size_t bytes = 3 * (size_t)n * dsize(dtype);
+    void* to[4] = {nullptr, nullptr, nullptr, nullptr};
+    bool any = false;
+    ffk::In4<ffk::vec4<R>> in;
+    ffk::Out4<double> out64;
+    ffk::Out4<float> out32;
+    for (int q = 0; q < 4; ++q) {
+        if (!dst[q]) continue;
+        any = true;
+        to[q] = loc == FF_HOST ? static_cast<char*>(c->staging) + (size_t)q * 3 * n * sizeof(double)
+                               : dst[q];
+        in.p[q] = static_cast<const ffk::vec4<R>*>(src[q]);
+        out64.p[q] = static_cast<double*>(to[q]);
+        out32.p[q] = static_cast<float*>(to[q]);
+    }
+    if (!any) return FF_OK;
+    {
+        StageTimer tm(c, S_OUT);
+        if (dtype == FF_DTYPE_F64)
+            ffk::scatter_state<R, double>(in, id, n, out64, c->stream);
+        else
+            ffk::scatter_state<R, float>(in, id, n, out32, c->stream);
+    }
     FF_LAUNCHED(c);
-    if (loc == FF_HOST)
-        FF_CUDA(c, cudaMemcpyAsync(dst, stg, 3 * n * dsize(dtype), cudaMemcpyDeviceToHost, c->stream));
+    for (int q = 0; q < 4; ++q)
+        if (dst[q] && loc == FF_HOST)
+            FF_CUDA(c, cudaMemcpyAsync(dst[q], to[q], bytes, cudaMemcpyDeviceToHost, c->stream));
     return FF_OK;
 }
 
@@ -793,12 +806,21 @@ ff_status get_particles(ff_ctx* c, void* pos, void* u, void* vel, void* om, int3
                         int32_t loc)
 {
     Buffers& a = c->st[c->cur];
-    ff_status s;
-    if ((s = store_array<R>(c, a.pos, a.id, pos, dtype, loc, 0)) != FF_OK) return s;
-    if ((s = store_array<R>(c, a.u, a.id, u, dtype, loc, 1)) != FF_OK) return s;
-    if ((s = store_array<R>(c, a.vel, a.id, vel, dtype, loc, 2)) != FF_OK) return s;
-    if ((s = store_array<R>(c, a.om, a.id, om, dtype, loc, 3)) != FF_OK) return s;
-    return sync_and_check(c);
+    const void* const src[4] = {a.pos, a.u, a.vel, a.om};
+    void* const dst[4] = {pos, u, vel, om};
+    const ff_status s = store_arrays<R>(c, src, dst, dtype, loc);
+    return s != FF_OK ? s : sync_and_check(c);
+}
+
+// Writes two record arrays (field and force, or the gradients) and waits.
+template <typename R>
+ff_status store_pair(ff_ctx* c, const void* a, void* a_out, const void* b, void* b_out,
+                     int32_t dtype, int32_t loc)
+{
+    const void* const src[4] = {a, b, nullptr, nullptr};
+    void* const dst[4] = {a_out, b_out, nullptr, nullptr};
+    const ff_status s = store_arrays<R>(c, src, dst, dtype, loc);
+    return s != FF_OK ? s : sync_and_check(c);
 }
 
 template <typename R>
@@ -807,10 +829,7 @@ ff_status dipolar_field(ff_ctx* c, int32_t algo, double theta, int32_t include_s
 {
     ff_status s = eval_field<R>(c, algo, theta, include_sr);
     if (s != FF_OK) return s;
-    const uint32_t* id = c->st[c->cur].id;
-    if ((s = store_array<R>(c, c->h, id, h_out, dtype, loc, 0)) != FF_OK) return s;
-    if ((s = store_array<R>(c, c->f, id, f_out, dtype, loc, 1)) != FF_OK) return s;
-    return sync_and_check(c);
+    return store_pair<R>(c, c->h, h_out, c->f, f_out, dtype, loc);
 }
 
 template <typename R>
@@ -1528,15 +1547,8 @@ ff_status ff_energy_grad(ff_ctx* c, int32_t algo, double theta, double* energy, 
         ff_status st = c->fp64 ? energy_grad<double>(c, algo, theta, energy, grads)
                                : energy_grad<float>(c, algo, theta, energy, grads);
         if (st != FF_OK || !grads) return st;
-        const uint32_t* id = c->st[c->cur].id;
-        if (c->fp64) {
-            if ((st = store_array<double>(c, c->g_pos, id, grad_pos, dtype, loc, 0)) != FF_OK) return st;
-            if ((st = store_array<double>(c, c->g_u, id, grad_u, dtype, loc, 1)) != FF_OK) return st;
-        } else {
-            if ((st = store_array<float>(c, c->g_pos, id, grad_pos, dtype, loc, 0)) != FF_OK) return st;
-            if ((st = store_array<float>(c, c->g_u, id, grad_u, dtype, loc, 1)) != FF_OK) return st;
-        }
-        return sync_and_check(c);
+        return c->fp64 ? store_pair<double>(c, c->g_pos, grad_pos, c->g_u, grad_u, dtype, loc)
+                       : store_pair<float>(c, c->g_pos, grad_pos, c->g_u, grad_u, dtype, loc);
     });
 }
 

@@ -467,11 +467,23 @@ void step_set(unsigned long long* step, unsigned long long v, cudaStream_t s);
 // records; scatter/gather through the particle ids.
 template <typename R, typename I>
 void load3(const I* in, int64_t n, vec4<R>* out, cudaStream_t s);
-template <typename R>
-void fill_zero4(vec4<R>* out, int64_t n, cudaStream_t s);
-void iota32(uint32_t* out, int64_t n, cudaStream_t s);
+// (four arrays at a time: positions, moments, velocities, angular velocities)
+template <typename T>
+struct In4 {
+    const T* p[4] = {nullptr, nullptr, nullptr, nullptr};
+};
+template <typename T>
+struct Out4 {
+    T* p[4] = {nullptr, nullptr, nullptr, nullptr};
+};
+// null inputs are zero; id[i] = i
+template <typename R, typename I>
+void load_state(const In4<I>& in, int64_t n, const Out4<vec4<R>>& out, uint32_t* id,
+                cudaStream_t s);
+// null outputs are left out
 template <typename R, typename O>
-void scatter3(const vec4<R>* in, const uint32_t* id, int64_t n, O* out, cudaStream_t s);
+void scatter_state(const In4<vec4<R>>& in, const uint32_t* id, int64_t n, const Out4<O>& out,
+                   cudaStream_t s);
 template <typename R>
 void scatter_counts(const int4* in, const uint32_t* id, int64_t n, int32_t* a, int32_t* p,
                     int32_t* o, cudaStream_t s);

@@ -334,33 +334,45 @@ __global__ void k_load3(const I* __restrict__ in, int64_t n, vec4<R>* __restrict
     out[i] = v;
 }
 
-template <typename R>
-__global__ void k_zero4(vec4<R>* __restrict__ out, int64_t n)
+// A whole state in one launch (positions, moments, velocities, angular
+// velocities; null: zero) and the particles' ids.  Five launches of a small state
+// took 12 us.
+template <typename R, typename I>
+__global__ void k_load_state(In4<I> in, int64_t n, Out4<vec4<R>> out, uint32_t* __restrict__ id)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    vec4<R> v;
-    v.x = v.y = v.z = v.w = R(0);
-    out[i] = v;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        vec4<R> v;
+        v.x = v.y = v.z = v.w = R(0);
+        if (in.p[q]) {
+            v.x = (R)in.p[q][3 * i];
+            v.y = (R)in.p[q][3 * i + 1];
+            v.z = (R)in.p[q][3 * i + 2];
+        }
+        out.p[q][i] = v;
+    }
+    id[i] = (uint32_t)i;
 }
 
-__global__ void k_iota(uint32_t* __restrict__ out, int64_t n)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = (uint32_t)i;
-}
-
+// Up to four record arrays to the caller's arrays in the caller's order (null
+// outputs are left out), one launch.
 template <typename R, typename O>
-__global__ void k_scatter3(const vec4<R>* __restrict__ in, const uint32_t* __restrict__ id,
-                           int64_t n, O* __restrict__ out)
+__global__ void k_scatter_state(In4<vec4<R>> in, const uint32_t* __restrict__ id, int64_t n,
+                                Out4<O> out)
 {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
-    const vec4<R> v = in[s];
     const int64_t d = id[s];
-    out[3 * d] = (O)v.x;
-    out[3 * d + 1] = (O)v.y;
-    out[3 * d + 2] = (O)v.z;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if (!out.p[q]) continue;
+        const vec4<R> v = in.p[q][s];
+        out.p[q][3 * d] = (O)v.x;
+        out.p[q][3 * d + 1] = (O)v.y;
+        out.p[q][3 * d + 2] = (O)v.z;
+    }
 }
 
 __global__ void k_scatter_counts(const int4* __restrict__ in, const uint32_t* __restrict__ id,
@@ -562,23 +574,18 @@ void load3(const I* in, int64_t n, vec4<R>* out, cudaStream_t s)
     counted();
 }
 
-template <typename R>
-void fill_zero4(vec4<R>* out, int64_t n, cudaStream_t s)
+template <typename R, typename I>
+void load_state(const In4<I>& in, int64_t n, const Out4<vec4<R>>& out, uint32_t* id, cudaStream_t s)
 {
-    k_zero4<R><<<nblk(n, 256), 256, 0, s>>>(out, n);
-    counted();
-}
-
-void iota32(uint32_t* out, int64_t n, cudaStream_t s)
-{
-    k_iota<<<nblk(n, 256), 256, 0, s>>>(out, n);
+    k_load_state<R, I><<<nblk(n, 256), 256, 0, s>>>(in, n, out, id);
     counted();
 }
 
 template <typename R, typename O>
-void scatter3(const vec4<R>* in, const uint32_t* id, int64_t n, O* out, cudaStream_t s)
+void scatter_state(const In4<vec4<R>>& in, const uint32_t* id, int64_t n, const Out4<O>& out,
+                   cudaStream_t s)
 {
-    k_scatter3<R, O><<<nblk(n, 256), 256, 0, s>>>(in, id, n, out);
+    k_scatter_state<R, O><<<nblk(n, 256), 256, 0, s>>>(in, id, n, out);
     counted();
 }
 
@@ -601,17 +608,19 @@ void scatter_counts(const int4* in, const uint32_t* id, int64_t n, int32_t* a, i
     template void observables<R>(int64_t, const vec4<R>*, const vec4<R>*, const vec4<R>*,        \
                                  const vec4<R>*, const vec4<R>*, const R*, DynParams<R>,         \
                                  double*, cudaStream_t);                                        \
-    template void load3<R, float>(const float*, int64_t, vec4<R>*, cudaStream_t);               \
-    template void load3<R, double>(const double*, int64_t, vec4<R>*, cudaStream_t);             \
-    template void fill_zero4<R>(vec4<R>*, int64_t, cudaStream_t);                               \
-    template void scatter3<R, float>(const vec4<R>*, const uint32_t*, int64_t, float*,           \
-                                     cudaStream_t);                                             \
-    template void scatter3<R, double>(const vec4<R>*, const uint32_t*, int64_t, double*,         \
-                                      cudaStream_t);                                            \
+    template void load_state<R, float>(const In4<float>&, int64_t, const Out4<vec4<R>>&,         \
+                                       uint32_t*, cudaStream_t);                               \
+    template void load_state<R, double>(const In4<double>&, int64_t, const Out4<vec4<R>>&,       \
+                                        uint32_t*, cudaStream_t);                              \
+    template void scatter_state<R, float>(const In4<vec4<R>>&, const uint32_t*, int64_t,         \
+                                          const Out4<float>&, cudaStream_t);                   \
+    template void scatter_state<R, double>(const In4<vec4<R>>&, const uint32_t*, int64_t,        \
+                                           const Out4<double>&, cudaStream_t);                 \
     template void scatter_counts<R>(const int4*, const uint32_t*, int64_t, int32_t*, int32_t*,   \
                                     int32_t*, cudaStream_t);
 FFK_INST(float)
 FFK_INST(double)
 #undef FFK_INST
+template void load3<float, float>(const float*, int64_t, float4*, cudaStream_t);
 
 }  // namespace ffk

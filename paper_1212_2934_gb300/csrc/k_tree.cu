@@ -560,7 +560,9 @@ __global__ void k_bbox_init(BBox* bb)
     }
 }
 
-// One block per system: extrema of the positions [start[s], start[s+1]).
+// One block per system: extrema of the positions [start[s], start[s+1]).  The
+// largest system's block is the launch (64 systems of up to 65,536 particles, keys
+// stage: 76 us with 256 threads, 44 with 1024).
 template <typename R>
 __global__ void k_bbox_seg(const vec4<R>* __restrict__ pos, const int* __restrict__ start,
                            BBox* bb, int* flags)
@@ -1282,7 +1284,7 @@ void morton_keys(const vec4<R>* pos, int64_t n, BBox* bb, uint64_t* keys, uint32
                  int* flags, Segs sg, cudaStream_t s)
 {
     if (sg.of_pos) {
-        k_bbox_seg<R><<<sg.nseg, 256, 0, s>>>(pos, sg.start, bb, flags);
+        k_bbox_seg<R><<<sg.nseg, 1024, 0, s>>>(pos, sg.start, bb, flags);
         counted();
     } else {
         k_bbox_init<<<1, 1, 0, s>>>(bb);
