@@ -851,7 +851,7 @@ def run_ours(args):
                         "pair_interactions_per_s": n * (n - 1) / (ap_field_ms / 1e3),
                         "field_tflops": n * (n - 1) * FLOPS_PER_INTERACTION / (ap_field_ms / 1e3) / 1e12},
             "bh_fp64": {"particle_steps_per_s": n / (ms64 / 1e3), "ms_per_step": ms64,
-                        "roofline": {"bound": "alu", "kernel": "k_bh<double> (FP64 traversal)",
+                        "roofline": {"bound": "alu", "kernel": "k_warp_walk64 (FP64 traversal)",
                                      "achieved": ach64, "peak": peaks["fp64_tflops"],
                                      "unit": "TFLOP/s", "frac": ach64 / peaks["fp64_tflops"],
                                      "avg_launch_ms": field64_ms,
@@ -1047,9 +1047,9 @@ def run_grad(args):
     f1.record(stream)
     barrier()
     field_ms = f0.elapsed_time(f1) / K
-    # roofline of the largest kernel, the counting walk that also writes the source lists
-    # (k_bh_rec): its launch time from the library's stage events over K more gradients,
-    # its work from the interaction counts of the same walk
+    # roofline of the largest kernel, the shared walk that also writes the tasks' records
+    # (k_warp_walk): its launch time from the library's stage events over K more gradients,
+    # its work from the interaction counts of the same evaluation
     ff.ff_profile(ctx, True)
     for _ in range(K):
         grad_once()
@@ -1066,12 +1066,11 @@ def run_grad(args):
     roofline = {"bound": "alu", "achieved": achieved, "peak": peaks["fp32_tflops"],
                 "unit": "TFLOP/s", "frac": achieved / peaks["fp32_tflops"],
                 "traffic": traffic_for(os.path.join(ROOT, "paper_1212_2934_gb300", "csrc",
-                                                    "k_field.cu"), n, "grad", args.theta,
-                                       args.leaf_max, 0, kernel="k_bh_rec"),
-                "kernel": "k_bh_rec (counting walk writing every particle's source list)",
+                                                    "k_walk.cu"), n, "grad", args.theta,
+                                       args.leaf_max, 0, kernel="k_warp_walk"),
+                "kernel": "k_warp_walk (shared walk writing every task's source records)",
                 "peak_note": peak_note(peaks, "fp32"), "peaks_measured": peaks,
                 "algorithmic_flops_per_launch": rec_flops,
-                "list_bytes_per_launch": 4.0 * inter,
                 "avg_launch_ms": rec_ms,
                 "timing": "CUDA events around the walk's launch on the library's stream, %d "
                           "gradients right after the timed region" % K}

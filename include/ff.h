@@ -139,7 +139,7 @@ void ff_params_default(ff_params *p);
 /*
  * Creates a context for p->n particles on p->device (Sec. 2 model, Sec. 3
  * schemes) and allocates its device memory: about 0.5 KB per particle in FP32
- * (0.6 KB up to 106,496 particles) and 0.8 KB in FP64 (66 GB and 110 GB at n = 2^27), gradient buffers apart.
+ * (0.6 KB up to 106,496 particles) and 0.9 KB in FP64 (66 GB and 119 GB at n = 2^27), gradient buffers apart.
  * The tree's cell arrays start with room for 2 n + 8192 cells (gases, chains
  * and dense packings use 1.2 to 1.8 cells per particle).  A build that needs
  * more raises a device flag instead of writing past them; that step and the
@@ -295,11 +295,13 @@ ff_status ff_tune_schedule(ff_ctx *ctx, int32_t reps, int32_t *best_schedule, fl
  * order); *energy (may be NULL) receives E in FP64; grad_pos and grad_u (may
  * be NULL) receive n x 3 values in the caller's order, dtype/loc as in
  * ff_get_particles.  With both NULL only the field and E are computed (the
- * cost of one field evaluation).  The Barnes-Hut gradient keeps every
- * particle's list of sources (4 bytes per interaction, in chunks of 128;
- * 700 to 900 interactions per particle at theta = 0.5) and 8 bytes per
- * interaction of record space, allocated on first use and grown as needed
- * (about 10 KB per particle in all at theta = 0.5); 2^32 - 16 interactions
+ * cost of one field evaluation).  The Barnes-Hut gradient of a
+ * single-precision context that does not count interactions keeps each source
+ * of 32 consecutive particles once (about 2 KB per particle in all at
+ * theta = 0.5); in FP64, or counting, it keeps every particle's list of sources
+ * (4 bytes per interaction, 700 to 900 interactions per particle at
+ * theta = 0.5) and 8 bytes per interaction of record space (about 10 KB per
+ * particle).  Both are allocated on first use and grown as needed; 2^32 - 16 interactions
  * or more (about 5 million particles at theta = 0.5) is FF_EINVAL.  Waits.
  */
 ff_status ff_energy_grad(ff_ctx *ctx, int32_t algo, double theta, double *energy, void *grad_pos,

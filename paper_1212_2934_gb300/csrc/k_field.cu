@@ -11,7 +11,9 @@
 // once per group (a broadcast load).  Large groups share more loads; small
 // groups waste fewer lane slots on cells only some lanes need.  Skip
 // pointers replace a stack.  Every lane's nxt strictly increases, so the
-// loop ends after at most ncells visits per group.
+// loop ends after at most ncells visits per group.  Small FP32 contexts
+// (k_walk.cu) and FP64 ones (k_walk64.cu) have walks of their own, which these
+// launchers choose by size, type and options.
 #include "walk.cuh"
 
 namespace ffk {

@@ -7,10 +7,13 @@
 //   dE/drho_k = -1/2 [ f_k - ds sum over (m, s), k in s, of
 //                      grad phi(rho_m - x_s; w_s, u_m) / n_s ]
 // h and f are the dipolar field and force of the same traversal (ds
-// included).  The reverse sums are formed without atomics.  The counting walk
-// writes every particle's sources (in depth-first order) to an entry pool; one
-// block per task of 32 consecutive particles gathers its 32 lists into records
-// (source, task, lane mask), one per source some lane takes; the records
+// included).  The reverse sums are formed without atomics.  A task of 32
+// consecutive particles has one record (source, task, lane mask) per source some
+// lane takes.  In single precision the walk of the task writes them as it goes
+// (k_walk.cu); in FP64, in contexts that count interactions and for the
+// vector-Jacobian product, the one-lane walk writes every particle's sources (in
+// depth-first order) to an entry pool and one block per task gathers its 32 lists
+// into records.  The records
 // (about a tenth as many as the (source, target) entries) are packed in task
 // order and sorted stably by source, so each source's entries, expanded lane
 // by lane, come out in target order.  Each source's entries are summed in a
