@@ -114,6 +114,48 @@ __global__ void k_scan_down(const uint32_t* __restrict__ in, int64_t n,
     }
 }
 
+// The same for few values in one launch of one block: thread t takes a run of
+// consecutive values.  The three launches of a small scan take 10 us; with this
+// one and the one-launch root cube below a field call of 1,000 particles went from
+// 321 to 315 us.
+constexpr int kSmallScanThreads = 1024;
+constexpr int64_t kSmallScanMax = 16384;
+
+__global__ void __launch_bounds__(kSmallScanThreads) k_scan_small(const uint32_t* __restrict__ in,
+                                                                  int n, uint32_t* __restrict__ out)
+{
+    __shared__ uint32_t ws[kSmallScanThreads / 32];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int per = (n + kSmallScanThreads - 1) / kSmallScanThreads;
+    const int b = min(t * per, n), e = min(b + per, n);
+    uint32_t s = 0;
+    for (int i = b; i < e; ++i) s += in[i];
+    uint32_t x = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) ws[w] = x;
+    __syncthreads();
+    if (w == 0) {
+        uint32_t v = ws[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(kFull, v, o);
+            if (lane >= o) v += y;
+        }
+        ws[lane] = v;
+    }
+    __syncthreads();
+    uint32_t ex = (w ? ws[w - 1] : 0u) + x - s;
+    for (int i = b; i < e; ++i) {
+        out[i] = ex;
+        ex += in[i];
+    }
+    if (t == kSmallScanThreads - 1) out[n] = ws[kSmallScanThreads / 32 - 1];
+}
+
 // ---------------------------------------------------- one-sweep radix sort
 // Digit of a sort element: 8 bits of its key at `shift` or, in a system pass
 // (sysd != null), of the system that owned the element's pre-sort position
@@ -565,13 +607,14 @@ __global__ void k_bbox_init(BBox* bb)
 // stage: 75 us with 256 threads, 40 with 1024).
 template <typename R>
 __global__ void k_bbox_seg(const vec4<R>* __restrict__ pos, const int* __restrict__ start,
-                           BBox* bb, int* flags)
+                           int64_t n, BBox* bb, int* flags)
 {
     const int sgi = blockIdx.x;
+    const int64_t first = start ? start[sgi] : 0, last = start ? start[sgi + 1] : n;
     long long lo[3] = {LLONG_MAX, LLONG_MAX, LLONG_MAX};
     long long hi[3] = {LLONG_MIN, LLONG_MIN, LLONG_MIN};
     bool bad = false;
-    for (int64_t i = start[sgi] + threadIdx.x; i < start[sgi + 1]; i += blockDim.x) {
+    for (int64_t i = first + threadIdx.x; i < last; i += blockDim.x) {
         vec4<R> p = pos[i];
         R c[3] = {p.x, p.y, p.z};
 #pragma unroll
@@ -1159,6 +1202,11 @@ size_t scan_tmp_words(int64_t n)
 
 void scan_exclusive(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* tmp, cudaStream_t s)
 {
+    if (n > 0 && n <= kSmallScanMax) {
+        k_scan_small<<<1, kSmallScanThreads, 0, s>>>(in, (int)n, out);
+        counted();
+        return;
+    }
     const int64_t nb = (n + kScanTile - 1) / kScanTile;
     if (nb > 0) k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, tmp);
     k_scan_top<<<1, kScanThreads, 0, s>>>(tmp, nb, out + n);
@@ -1284,7 +1332,11 @@ void morton_keys(const vec4<R>* pos, int64_t n, BBox* bb, uint64_t* keys, uint32
                  int* flags, Segs sg, cudaStream_t s)
 {
     if (sg.of_pos) {
-        k_bbox_seg<R><<<sg.nseg, 1024, 0, s>>>(pos, sg.start, bb, flags);
+        k_bbox_seg<R><<<sg.nseg, 1024, 0, s>>>(pos, sg.start, n, bb, flags);
+        counted();
+    } else if (n <= 8192) {
+        // few particles: one block, without the launch that prepares the atomics
+        k_bbox_seg<R><<<1, 1024, 0, s>>>(pos, nullptr, n, bb, flags);
         counted();
     } else {
         k_bbox_init<<<1, 1, 0, s>>>(bb);
