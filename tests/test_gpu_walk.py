@@ -157,3 +157,20 @@ def test_gradient_records_match_lists(ff, n, leaf_max):
         res[-1] += tuple(ff.ff_get_particles(ctx))
     for a, b in zip(*res):
         assert np.array_equal(a, b)
+
+
+def test_gradient_records_outgrow_their_pool(ff):
+    """At a small opening angle a task's records need more chunks than the pool's first
+    allocation (6000 particles, nearly all of them a source of each task: 17,600 chunks against
+    10,024): the walk is redone with room for what it took, and the result is that of a second
+    call and of the lists."""
+    pos, u = _gas(6000, 17)
+    res = []
+    for count in (0, 1):
+        ctx = ff.ff_create(ff.ff_params_default(n=6000, count_interactions=count))
+        ff.ff_set_particles(ctx, pos, u)
+        for _ in range(2):
+            res.append(ff.ff_energy_grad(ctx, ff.FF_ALGO_BH, 0.05, dtype=np.float32))
+    for r in res[1:]:
+        assert r[0] == res[0][0]
+        assert np.array_equal(r[1], res[0][1]) and np.array_equal(r[2], res[0][2])
