@@ -722,35 +722,39 @@ constexpr int kAp2Pair = 20;           // words per staged pair (14 used)
 constexpr int kAp2Stage = 16 * kAp2Pair + 4;
 constexpr int64_t kApWide = 65536;
 
-template <int T>
-__global__ void __launch_bounds__(32 * kAp2Warps, 2) k_ap2(const float4* __restrict__ pos,
-                                                           const float4* __restrict__ u, int n,
-                                                           FieldParams<float> fp,
-                                                           float4* __restrict__ h,
-                                                           float4* __restrict__ f,
-                                                           float* __restrict__ esr)
+// A target (each value twice) and its sums (two sources at a time, kept apart).
+struct Ap2Target {
+    float2 x, y, z, ux, uy, uz;
+};
+struct Ap2Sums {
+    float2 hx, hy, hz, fx, fy, fz;
+    float sx, sy, sz, es;
+};
+
+// This warp's share of the sources on its targets.  A source at r^2 = 0 (the
+// target itself, a coincident particle) or at an undefined one (a position that
+// is not a number) adds nothing.  1/r = 0 sees to that as long as the rest of
+// its terms is finite; EXACT leaves the terms out one by one instead, whatever
+// they are, and gives sources past the end an undefined position.
+template <int T, bool EXACT>
+__device__ __forceinline__ void ap2_sweep(const float4* __restrict__ pos,
+                                          const float4* __restrict__ u, int n,
+                                          const FieldParams<float>& fp, float* stage,
+                                          const Ap2Target& k, Ap2Sums& a)
 {
-    constexpr int kGroups = 32 / T;         // groups of T lanes in a warp
-    constexpr int kPairs = 16 / kGroups;    // staged pairs of each
-    constexpr int kSums = 10;
-    __shared__ __align__(16) float sm[kAp2Warps * kAp2Stage];
-    static_assert(kAp2Warps * kAp2Stage >= kAp2Warps * 32 * kSums, "room for the partial sums");
+    constexpr int kPairs = 16 / (32 / T);  // staged pairs of each group of T lanes
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, grp = lane / T;
-    const int k = blockIdx.x * T + lane % T;
-    const float4 xk = pos[min(k, n - 1)], uk = u[min(k, n - 1)];
-    float* stage = sm + w * kAp2Stage;
     // (the second group's pairs start 4 words on: other banks)
     float* mine = stage + (lane >> 1) * kAp2Pair + (lane & 1) + ((lane >> 1) >= kPairs ? 4 : 0);
     const float* own = stage + grp * (kPairs * kAp2Pair + 4);
-    const float2 kx = dup2(xk.x), ky = dup2(xk.y), kz = dup2(xk.z);
-    const float2 ux = dup2(uk.x), uy = dup2(uk.y), uz = dup2(uk.z);
     const float2 zero = dup2(0.0f);
     float2 thx = zero, thy = zero, thz = zero, tfx = zero, tfy = zero, tfz = zero;
     float2 hx = zero, hy = zero, hz = zero, fx = zero, fy = zero, fz = zero;
     float sx = 0.0f, sy = 0.0f, sz = 0.0f, es = 0.0f;
     const float near2 = fp.include_sr ? fp.lj_rcut2_hi : 0.0f;
     // past the end: no moment, far away
-    const float4 none = make_float4(1e18f, 1e18f, 1e18f, 0.0f);
+    const float far = EXACT ? __int_as_float(0x7fffffff) : 1e18f;
+    const float4 none = make_float4(far, far, far, 0.0f);
     int j = w * 32 + lane;
     float4 c = j < n ? pos[j] : none, m = j < n ? u[j] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     for (int base = w * 32, it = 1; base < n; base += 32 * kAp2Warps, ++it) {
@@ -770,34 +774,36 @@ __global__ void __launch_bounds__(32 * kAp2Warps, 2) k_ap2(const float4* __restr
 #pragma unroll 2
         for (int p = 0; p < kPairs; ++p, q += kAp2Pair / 4) {
             const float4 q0 = q[0], q1 = q[1], q2 = q[2];
-            const float2 rx = __fadd2_rn(kx, make_float2(q0.x, q0.y));
-            const float2 ry = __fadd2_rn(ky, make_float2(q0.z, q0.w));
-            const float2 rz = __fadd2_rn(kz, make_float2(q1.x, q1.y));
+            const float2 rx = __fadd2_rn(k.x, make_float2(q0.x, q0.y));
+            const float2 ry = __fadd2_rn(k.y, make_float2(q0.z, q0.w));
+            const float2 rz = __fadd2_rn(k.z, make_float2(q1.x, q1.y));
             const float2 vx = make_float2(q1.z, q1.w), vy = make_float2(q2.x, q2.y),
                          vz = make_float2(q2.z, q2.w);
             const float2 r2 = pair_r2_2(rx, ry, rz);
-            // the target itself, and coincident particles, add nothing
-            const float2 ir = make_float2(r2.x > 0.0f ? dip_rsqrt(r2.x) : 0.0f,
-                                          r2.y > 0.0f ? dip_rsqrt(r2.y) : 0.0f);
+            const bool in0 = r2.x > 0.0f, in1 = r2.y > 0.0f;
+            const auto kept = [&](float2 v) {
+                return EXACT ? make_float2(in0 ? v.x : 0.0f, in1 ? v.y : 0.0f) : v;
+            };
+            const float2 ir = make_float2(in0 ? dip_rsqrt(r2.x) : 0.0f, in1 ? dip_rsqrt(r2.y) : 0.0f);
             const float2 ir2 = __fmul2_rn(ir, ir);
             const float2 ir3 = __fmul2_rn(ir2, ir);
             const float2 p3 = __fmul2_rn(dup2(3.0f), ir2);
             const float2 bj = __ffma2_rn(vz, rz, __ffma2_rn(vy, ry, __fmul2_rn(vx, rx)));
-            const float2 bk = __ffma2_rn(uz, rz, __ffma2_rn(uy, ry, __fmul2_rn(ux, rx)));
-            const float2 a = __ffma2_rn(vz, uz, __ffma2_rn(vy, uy, __fmul2_rn(vx, ux)));
+            const float2 bk = __ffma2_rn(k.uz, rz, __ffma2_rn(k.uy, ry, __fmul2_rn(k.ux, rx)));
+            const float2 ab = __ffma2_rn(vz, k.uz, __ffma2_rn(vy, k.uy, __fmul2_rn(vx, k.ux)));
             // h += [3 r (u_j.r) / r^2 - u_j] / r^3
             const float2 qh = __fmul2_rn(p3, bj);
             const float2 nir3 = make_float2(-ir3.x, -ir3.y);
             const float2 nqh = make_float2(-qh.x, -qh.y);
-            thx = __ffma2_rn(nir3, __ffma2_rn(rx, nqh, vx), thx);
-            thy = __ffma2_rn(nir3, __ffma2_rn(ry, nqh, vy), thy);
-            thz = __ffma2_rn(nir3, __ffma2_rn(rz, nqh, vz), thz);
+            thx = __ffma2_rn(nir3, kept(__ffma2_rn(rx, nqh, vx)), thx);
+            thy = __ffma2_rn(nir3, kept(__ffma2_rn(ry, nqh, vy)), thy);
+            thz = __ffma2_rn(nir3, kept(__ffma2_rn(rz, nqh, vz)), thz);
             // f += 3 / r^5 {r [u_j.u_k - 5 (u_k.r)(u_j.r) / r^2] + u_k (u_j.r) + u_j (u_k.r)}
             const float2 g = __fmul2_rn(p3, ir3);
-            const float2 wv = __ffma2_rn(__fmul2_rn(dup2(-5.0f), ir2), __fmul2_rn(bj, bk), a);
-            tfx = __ffma2_rn(g, __ffma2_rn(rx, wv, __ffma2_rn(ux, bj, __fmul2_rn(vx, bk))), tfx);
-            tfy = __ffma2_rn(g, __ffma2_rn(ry, wv, __ffma2_rn(uy, bj, __fmul2_rn(vy, bk))), tfy);
-            tfz = __ffma2_rn(g, __ffma2_rn(rz, wv, __ffma2_rn(uz, bj, __fmul2_rn(vz, bk))), tfz);
+            const float2 wv = __ffma2_rn(__fmul2_rn(dup2(-5.0f), ir2), __fmul2_rn(bj, bk), ab);
+            tfx = __ffma2_rn(g, kept(__ffma2_rn(rx, wv, __ffma2_rn(k.ux, bj, __fmul2_rn(vx, bk)))), tfx);
+            tfy = __ffma2_rn(g, kept(__ffma2_rn(ry, wv, __ffma2_rn(k.uy, bj, __fmul2_rn(vy, bk)))), tfy);
+            tfz = __ffma2_rn(g, kept(__ffma2_rn(rz, wv, __ffma2_rn(k.uz, bj, __fmul2_rn(vz, bk)))), tfz);
             if (r2.x < near2) close |= one;
             if (r2.y < near2) close |= one << 1;
             one <<= 2;
@@ -807,7 +813,7 @@ __global__ void __launch_bounds__(32 * kAp2Warps, 2) k_ap2(const float4* __restr
             const int b = __ffs(close) - 1;
             close &= close - 1u;
             const float* st = own + (b >> 1) * kAp2Pair + (b & 1);
-            const float rx = xk.x + st[0], ry = xk.y + st[2], rz = xk.z + st[4];
+            const float rx = k.x.x + st[0], ry = k.y.x + st[2], rz = k.z.x + st[4];
             lj<float>(fp, rx, ry, rz, pair_r2(rx, ry, rz), sx, sy, sz, es);
         }
         if ((it & 7) == 0) {
@@ -816,13 +822,63 @@ __global__ void __launch_bounds__(32 * kAp2Warps, 2) k_ap2(const float4* __restr
             thx = thy = thz = tfx = tfy = tfz = zero;
         }
     }
-    hx = __fadd2_rn(hx, thx); hy = __fadd2_rn(hy, thy); hz = __fadd2_rn(hz, thz);
-    fx = __fadd2_rn(fx, tfx); fy = __fadd2_rn(fy, tfy); fz = __fadd2_rn(fz, tfz);
+    a.hx = __fadd2_rn(hx, thx); a.hy = __fadd2_rn(hy, thy); a.hz = __fadd2_rn(hz, thz);
+    a.fx = __fadd2_rn(fx, tfx); a.fy = __fadd2_rn(fy, tfy); a.fz = __fadd2_rn(fz, tfz);
+    a.sx = sx; a.sy = sy; a.sz = sz; a.es = es;
+}
+
+// A lane's sums to its place among the block's.
+__device__ __forceinline__ void ap2_store(const Ap2Sums& a, float* r)
+{
+    r[0] = a.hx.x + a.hx.y; r[1] = a.hy.x + a.hy.y; r[2] = a.hz.x + a.hz.y;
+    r[3] = a.fx.x + a.fx.y; r[4] = a.fy.x + a.fy.y; r[5] = a.fz.x + a.fz.y;
+    r[6] = a.sx; r[7] = a.sy; r[8] = a.sz; r[9] = a.es;
+}
+
+// A block whose sums hold an undefined value forms them again with EXACT: zero
+// times an infinite or undefined term (a moment that is not finite or too large for
+// products of two, an undefined position) is undefined and stays so in a sum, so
+// nothing is missed, and the test costs other blocks one barrier vote.  (Leaving
+// terms out in every pair cost 8 %: n = 65,536 6.78 -> 7.46 ms; in line rather than
+// as a call, this code cost 1.5 us of the 74 of a field call at n = 1,000.)
+template <int T>
+__device__ __noinline__ void ap2_exact(const float4* __restrict__ pos, const float4* __restrict__ u,
+                                       int n, const FieldParams<float>& fp, float* stage, float4 xk,
+                                       float4 uk, float* r)
+{
+    const Ap2Target tg = {dup2(xk.x), dup2(xk.y), dup2(xk.z), dup2(uk.x), dup2(uk.y), dup2(uk.z)};
+    Ap2Sums a;
+    ap2_sweep<T, true>(pos, u, n, fp, stage, tg, a);
     __syncthreads();
+    ap2_store(a, r);
+}
+
+template <int T>
+__global__ void __launch_bounds__(32 * kAp2Warps, 2) k_ap2(const float4* __restrict__ pos,
+                                                           const float4* __restrict__ u, int n,
+                                                           FieldParams<float> fp,
+                                                           float4* __restrict__ h,
+                                                           float4* __restrict__ f,
+                                                           float* __restrict__ esr)
+{
+    constexpr int kGroups = 32 / T;         // groups of T lanes in a warp
+    constexpr int kSums = 10;
+    __shared__ __align__(16) float sm[kAp2Warps * kAp2Stage];
+    static_assert(kAp2Warps * kAp2Stage >= kAp2Warps * 32 * kSums, "room for the partial sums");
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int k = blockIdx.x * T + lane % T;
+    const float4 xk = pos[min(k, n - 1)], uk = u[min(k, n - 1)];
+    const Ap2Target tg = {dup2(xk.x), dup2(xk.y), dup2(xk.z), dup2(uk.x), dup2(uk.y), dup2(uk.z)};
+    float* stage = sm + w * kAp2Stage;
     float* r = sm + (w * 32 + lane) * kSums;
-    r[0] = hx.x + hx.y; r[1] = hy.x + hy.y; r[2] = hz.x + hz.y;
-    r[3] = fx.x + fx.y; r[4] = fy.x + fy.y; r[5] = fz.x + fz.y;
-    r[6] = sx; r[7] = sy; r[8] = sz; r[9] = es;
+    Ap2Sums a;
+    ap2_sweep<T, false>(pos, u, n, fp, stage, tg, a);
+    const float2 all = __fadd2_rn(__fadd2_rn(__fadd2_rn(a.hx, a.hy), __fadd2_rn(a.hz, a.fx)),
+                                  __fadd2_rn(a.fy, a.fz));
+    if (__syncthreads_or(isnan(all.x + all.y)))
+        ap2_exact<T>(pos, u, n, fp, stage, xk, uk, r);
+    else
+        ap2_store(a, r);
     __syncthreads();
     // component q of target t: the groups' sums in order
     for (int e = threadIdx.x; e < T * kSums; e += 32 * kAp2Warps) {

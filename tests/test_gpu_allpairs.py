@@ -74,3 +74,38 @@ def test_coincident_and_single(ff):
         hs, fs = ff.ff_dipolar_field(c, ff.FF_ALGO_AP, 0.0, True)
         np.testing.assert_allclose(h[k], hs[0], rtol=1e-5, atol=1e-5 * np.abs(hs).max())
         np.testing.assert_allclose(f[k], fs[0], rtol=1e-5, atol=1e-5 * np.abs(fs).max())
+
+
+@pytest.mark.parametrize("n", [1, 40, 600, 65569])
+@pytest.mark.parametrize("case", ["nan position", "infinite moment", "nan moment", "huge moment"])
+def test_undefined_and_huge_inputs(ff, n, case):
+    """What adds nothing adds nothing whatever its numbers are, as in double precision: a source
+    at an undefined distance (a position that is not a number, for the others and for itself),
+    and the target itself (its own moment infinite, undefined, or so large that its square
+    overflows).  The defined values agree with double precision within the bar."""
+    pos, u = _system(n, 5)
+    bad = [0] if n == 1 else [7, n // 2, n - 1]
+    if case == "nan position":
+        pos[bad[0], 1] = np.nan
+        pos[bad[-1]] = np.nan
+    elif case == "infinite moment":
+        u[bad[0]] = [0.0, np.inf, 0.0]
+    elif case == "nan moment":
+        u[bad[0], 2] = np.nan
+    else:
+        u[bad[0]] *= np.float32(1e25)
+    out = []
+    for prec, dt in (("f32", np.float32), ("f64", np.float64)):
+        ctx = ff.ff_create(ff.ff_params_default(n=n, algo="ap", precision=prec, lj_eps=0.0))
+        ff.ff_set_particles(ctx, pos.astype(dt), u.astype(dt))
+        out.append(ff.ff_dipolar_field(ctx, ff.FF_ALGO_AP, 0.0, True, dtype=dt))
+    (h, f), (h64, f64) = out
+    for a, b in ((h, h64), (f, f64)):
+        ok = np.isfinite(b)
+        assert np.array_equal(np.isfinite(a), ok)
+        rows = ok.all(axis=1)
+        none = rows & ~b.any(axis=1)
+        assert not a[none].any()
+        rows &= ~none
+        if rows.any():
+            assert _err(a[rows].astype(np.float64), b[rows]) <= 1e-5
