@@ -163,11 +163,12 @@ __device__ __forceinline__ void walk_pair(float rx, float ry, float rz, float r2
                                           float& hx, float& hy, float& hz, float& fx, float& fy,
                                           float& fz, float&)
 {
-    if (!(r2 > 0.0f)) return;
-    if (QUAD)
-        dipole<float>(rx, ry, rz, r2, ukx, uky, ukz, ujx, ujy, ujz, hx, hy, hz, fx, fy, fz);
-    else
+    if (QUAD) {
+        if (r2 > 0.0f)
+            dipole<float>(rx, ry, rz, r2, ukx, uky, ukz, ujx, ujy, ujz, hx, hy, hz, fx, fy, fz);
+    } else if (r2 > 0.0f) {
         walk_dipole<float>(rx, ry, rz, r2, ukx, uky, ukz, ujx, ujy, ujz, hx, hy, hz, fx, fy, fz);
+    }
 }
 
 template <bool QUAD>

@@ -95,9 +95,10 @@ constexpr int kTraverseCarveout = FFK_TRAVERSE_CARVEOUT;
 // taking 32 x its registers), so 128 x 10 allows 48 registers a thread, room
 // for the whole walk without spills.  The plain FP32 walk is lean enough for
 // 128 x 12 (40 registers, 48 warps) with a few spilled words, and measures
-// slightly faster so; the counting walk keeps 10 blocks, and the walk with
-// dipole-position terms 8 (64 registers, no spills; 131,071 particles at theta
-// 0.7: 0.627 ms, against 0.633 with 10).
+// slightly faster so; the other walks keep 10 blocks.  The walk with
+// dipole-position terms gains from more registers (54 a thread with 8 blocks asked
+// for, 36 warps an SM) only while all of its tasks are resident at once, where
+// fewer warps cost nothing: see bh_launch().
 #ifndef FFK_BH_THREADS
 #define FFK_BH_THREADS 128
 #endif
@@ -109,6 +110,7 @@ constexpr int kTraverseCarveout = FFK_TRAVERSE_CARVEOUT;
 #endif
 constexpr int kBhThreads = FFK_BH_THREADS;
 constexpr int kBhMinBlocks = FFK_BH_MIN_BLOCKS;
+constexpr int kBhMinBlocksQuadFew = 8;
 
 // FP64 walks hold twice the registers per value.
 #ifndef FFK_BH_MIN_BLOCKS_FP64
@@ -119,8 +121,7 @@ template <typename R, bool COUNT, bool QUAD>
 constexpr int bh_min_blocks()
 {
     return sizeof(R) == 8 ? FFK_BH_MIN_BLOCKS_FP64
-           : QUAD ? 8
-           : !COUNT ? FFK_BH_MIN_BLOCKS_LEAN
+           : (!COUNT && !QUAD) ? FFK_BH_MIN_BLOCKS_LEAN
                                : FFK_BH_MIN_BLOCKS;
 }
 static_assert(kBhThreads % 32 == 0, "whole warps");
@@ -899,9 +900,10 @@ __global__ void __launch_bounds__(32 * kAp2Warps, 2) k_ap2(const float4* __restr
 
 }  // namespace
 
+// RESIDENT: only where every task finds a warp at once (else false, and no launch).
 template <typename R, bool COUNT, int G, bool QUAD = false, int THREADS = kBhThreads,
-          int MINB = bh_min_blocks<R, COUNT, QUAD>()>
-void bh_launch_g(const vec4<R>* pos, const vec4<R>* u, int64_t n, Tree<R> t, FieldParams<R> fp,
+          int MINB = bh_min_blocks<R, COUNT, QUAD>(), bool RESIDENT = false>
+bool bh_launch_g(const vec4<R>* pos, const vec4<R>* u, int64_t n, Tree<R> t, FieldParams<R> fp,
                  vec4<R>* h, vec4<R>* f, R* esr, int4* counts, int* flags, int* work,
                  const uint32_t* off, Segs sg, cudaStream_t s)
 {
@@ -917,9 +919,11 @@ void bh_launch_g(const vec4<R>* pos, const vec4<R>* u, int64_t n, Tree<R> t, Fie
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, THREADS, 0);
         return per_sm;
     });
+    if (RESIDENT && (n + 31) / 32 > (int64_t)g.blocks * (THREADS / 32)) return false;
     cudaMemsetAsync(work, 0, sizeof(int) * g.nseg, s);
     kern<<<g.blocks, THREADS, 0, s>>>(pos, u, (int)n, t, fp, h, f, esr, counts, flags, work,
                                       g.nseg, off, sg);
+    return true;
 }
 
 template <typename R, bool COUNT>
@@ -965,9 +969,16 @@ void bh_launch(const vec4<R>* pos, const vec4<R>* u, int64_t n, Tree<R> t, Field
     } else {
     if (sched >= 1 && sched <= kNumSchedules) group = kSchedules[sched - 1].group;
     if (t.q1) {
-        // the dipole-position terms are evaluated by the one-lane walk only
-        bh_launch_g<R, COUNT, 1, true>(pos, u, n, t, fp, h, f, esr, counts, flags, work, off, sg,
-                                       s);
+        // the dipole-position terms are evaluated by the one-lane walk only.  While every
+        // task has a warp at once (to 175,104 particles: 54 registers, 36 warps on each
+        // of 152 SMs) it takes the shape with more registers; beyond, the 40 warps of the
+        // other hide more of its loads.  Field calls, ms with 10 / 8 blocks: 131,071
+        // particles at theta 0.7 0.976 / 0.940; 200,000 at 0.5 2.13 / 2.33; 1,048,576 at
+        // 0.7 4.47 / 4.65, at 0.5 9.60 / 9.77.
+        if (!bh_launch_g<R, COUNT, 1, true, kBhThreads, kBhMinBlocksQuadFew, true>(
+                pos, u, n, t, fp, h, f, esr, counts, flags, work, off, sg, s))
+            bh_launch_g<R, COUNT, 1, true>(pos, u, n, t, fp, h, f, esr, counts, flags, work, off,
+                                           sg, s);
         return;
     }
 #define FFK_BH_CASE(G) bh_launch_g<R, COUNT, G>(pos, u, n, t, fp, h, f, esr, counts, flags, work, off, sg, s)
