@@ -256,8 +256,9 @@ ff_status ff_tune_traversal(ff_ctx *ctx, const int32_t *groups, int32_t ngroups,
  * default shape, and the plain single-precision walk of up to 106,496 particles
  * has one shape of its own whatever the schedule.  The traversal is persistent (as many blocks as fit), so the
  * shape trades registers per thread against resident warps.  Every schedule
- * gives bit-identical fields and forces (each lane decides and sums for its own
- * particle in depth-first order).  ff_schedule_info fills the three numbers
+ * gives bit-identical fields and forces (in single precision each particle's
+ * sources are added in depth-first order; in double precision they go in turn,
+ * in that order, to four partial sums).  ff_schedule_info fills the three numbers
  * (any pointer may be NULL); FF_EINVAL for an index out of range.
  */
 int32_t ff_schedule_count(void);

@@ -64,12 +64,15 @@ __device__ __forceinline__ void source_of(uint32_t s, const Tree<double>& t,
     m = (s & kParticle) ? u[i] : t.mom[i];
 }
 
-// Sums the particles' lists: lane sub of a particle's lanes takes entries sub,
-// sub + 4, ... of its n.  LJ pairs (and, counting, the decision of one-particle
+// Sums the particles' lists, the n entries after the particle's first done: lane
+// sub of its lanes takes the entries that are sub, sub + 4, ... of all its sources,
+// so where the lists are cut, which the longest of the warp's decides, does not
+// matter.  LJ pairs (and, counting, the decision of one-particle
 // leaves) are left to the end of each 32 entries, so that one lane's pair does
 // not hold up the others at every entry.
 template <bool COUNT>
-__device__ __forceinline__ void sum_lists(const Walk64Shared& w, int n, const Tree<double>& t,
+__device__ __forceinline__ void sum_lists(const Walk64Shared& w, int n, int& done,
+                                          const Tree<double>& t,
                                           const FieldParams<double>& fp,
                                           const dvec4* __restrict__ pos,
                                           const dvec4* __restrict__ u, const dvec4& xk,
@@ -78,11 +81,13 @@ __device__ __forceinline__ void sum_lists(const Walk64Shared& w, int n, const Tr
     const int lane = threadIdx.x & 31, g = lane / kSub, sub = lane % kSub;
     const int most = __reduce_max_sync(kFull, n);
     __syncwarp();
-    for (int b = sub; b - sub < most; b += 32 * kSub) {
+    const int first = (sub - done) & (kSub - 1);
+    done += n;
+    for (int b = first; b - first < most; b += 32 * kSub) {
         uint32_t close = 0u;
         for (int r = 0; r < 32; ++r) {
             const int i = b + r * kSub;
-            if (i - sub >= most) break;
+            if (i - first >= most) break;
             if (i < n) {
                 const uint32_t s = w.src[g][i];
                 dvec4 c, m;
@@ -177,7 +182,7 @@ __device__ __forceinline__ void walk64_task(Walk64Shared& w, int task,
     const float ext2 = -warp_min(-(xf * xf + yf * yf + zf * zf));
     const float th2 = (float)fp.theta2, rcut2 = fp.use_rcut ? (float)fp.rcut2 : -3.0e38f;
     Sums64 a = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0, 0};
-    int nopen = 0, mine = 0, top = 0;
+    int nopen = 0, mine = 0, done = 0, top = 0;
     // the roots of the task's systems, the first on top
     __syncwarp();
     {
@@ -216,7 +221,7 @@ __device__ __forceinline__ void walk64_task(Walk64Shared& w, int task,
                 w.q.list[lane] = make_uint2((uint32_t)s | kParticle, mask);
                 hand_out(w, 32, lane, lt, mine);
                 if (__reduce_max_sync(kFull, mine) > kCap - 32) {
-                    sum_lists<COUNT>(w, mine, t, fp, pos, u, xk, uk, a);
+                    sum_lists<COUNT>(w, mine, done, t, fp, pos, u, xk, uk, a);
                     mine = 0;
                 }
             }
@@ -336,7 +341,7 @@ __device__ __forceinline__ void walk64_task(Walk64Shared& w, int task,
         }
         hand_out(w, emit, lane, lt, mine);
         if (__reduce_max_sync(kFull, mine) > kCap - 32) {
-            sum_lists<COUNT>(w, mine, t, fp, pos, u, xk, uk, a);
+            sum_lists<COUNT>(w, mine, done, t, fp, pos, u, xk, uk, a);
             mine = 0;
         }
         if (++rounds > max_rounds) {  // a damaged tree
@@ -344,7 +349,7 @@ __device__ __forceinline__ void walk64_task(Walk64Shared& w, int task,
             break;
         }
     }
-    sum_lists<COUNT>(w, mine, t, fp, pos, u, xk, uk, a);
+    sum_lists<COUNT>(w, mine, done, t, fp, pos, u, xk, uk, a);
     a.hx = group_sum(a.hx); a.hy = group_sum(a.hy); a.hz = group_sum(a.hz);
     a.fx = group_sum(a.fx); a.fy = group_sum(a.fy); a.fz = group_sum(a.fz);
     a.sx = group_sum(a.sx); a.sy = group_sum(a.sy); a.sz = group_sum(a.sz);

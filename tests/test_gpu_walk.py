@@ -137,6 +137,31 @@ def test_fp64_tasks_spanning_systems(ff):
 
 
 @pytest.mark.parametrize("leaf_max", [1, 6])
+def test_fp64_long_lists_do_not_depend_on_neighbours(ff, leaf_max):
+    """A particle's sources are summed 480 to 512 at a time, all of a warp's particles when the
+    longest list is full; which of its four partial sums a source goes to does not depend on that.
+    Systems whose lists are cut several times, at offsets that put other particles in the warps,
+    have the bits they have alone."""
+    sizes = [3001, 1500, 2503, 7, 1999]
+    parts = [_gas(k, 60 + k) for k in sizes]
+    pos = np.concatenate([p for p, _ in parts]).astype(np.float64)
+    u = np.concatenate([q for _, q in parts]).astype(np.float64)
+    (hp, fp), (hc, fc) = _both(ff, pos, u, 0.3, sizes=sizes, precision="f64", leaf_max=leaf_max,
+                               dtype=np.float64)
+    assert np.array_equal(hp, hc) and np.array_equal(fp, fc)
+    off = 0
+    for k, (p, q) in zip(sizes, parts):
+        ctx = ff.ff_create(ff.ff_params_default(n=k, precision="f64", leaf_max=leaf_max,
+                                                count_interactions=1))
+        ff.ff_set_particles(ctx, p.astype(np.float64), q.astype(np.float64))
+        h, f = ff.ff_dipolar_field(ctx, ff.FF_ALGO_BH, 0.3, True)
+        assert np.array_equal(h, hp[off:off + k]) and np.array_equal(f, fp[off:off + k])
+        acc, pairs, _ = ff.ff_get_counts(ctx)
+        assert k < 100 or (acc + pairs).max() > 512  # longer than a list
+        off += k
+
+
+@pytest.mark.parametrize("leaf_max", [1, 6])
 @pytest.mark.parametrize("n", [1, 31, 33, 3001, 120011])
 def test_gradient_records_match_lists(ff, n, leaf_max):
     """The gradient from the shared walk's records and from the lists of the counting walk (a
