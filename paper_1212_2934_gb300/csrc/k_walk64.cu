@@ -180,7 +180,12 @@ __device__ __forceinline__ void walk64_task(Walk64Shared& w, int task,
     const float lx = warp_min(xf), ly = warp_min(yf), lz = warp_min(zf);
     const float ux = -warp_min(-xf), uy = -warp_min(-yf), uz = -warp_min(-zf);
     const float ext2 = -warp_min(-(xf * xf + yf * yf + zf * zf));
-    const float th2 = (float)fp.theta2, rcut2 = fp.use_rcut ? (float)fp.rcut2 : -3.0e38f;
+    // quick decisions up to theta = 10, where a cube that may be accepted has its corners
+    // within 20 distances of its centre, and so their rounding within the slack; no quick
+    // one holds beyond (nor for angles whose square is no normal single-precision number)
+    const bool quick = fp.theta2 <= 100.0 && !(fp.theta2 > 0.0 && fp.theta2 < 1e-37);
+    const float th2 = quick ? (float)fp.theta2 : __int_as_float(0x7fffffff);
+    const float rcut2 = quick && fp.use_rcut ? (float)fp.rcut2 : -3.0e38f;
     Sums64 a = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0, 0};
     int nopen = 0, mine = 0, done = 0, top = 0;
     // the roots of the task's systems, the first on top

@@ -161,6 +161,35 @@ def test_fp64_long_lists_do_not_depend_on_neighbours(ff, leaf_max):
         off += k
 
 
+@pytest.mark.parametrize("theta", [1e-19, 0.5, 9.0, 11.0, 1e6, 1e25])
+def test_fp64_decides_exactly_at_any_angle(ff, theta):
+    """Particles about the LJ cut away from the upper face of a cube a million wide, whose own
+    particles lie at that face: at opening angles that accept it, the distance from its cube
+    decides, and the far corner it is formed from is a million away."""
+    import oracle
+    from conftest import rel_err
+
+    s = 2.0 ** 20
+    k = np.arange(64)
+    pos = np.zeros((68, 3))
+    pos[0, 1:] = s
+    pos[1, 0] = s
+    pos[2:4] = [[s / 2 - 0.3, 5000.0, 4000.0], [s / 2 - 0.4, 5003.0, 4001.0]]
+    pos[4:, 0] = s / 2 + 2.4 + 0.2 * k / 63
+    pos[4:, 1] = 4900.0 + 3.1 * k
+    pos[4:, 2] = 4000.0 + 0.7 * (k % 5)
+    u = np.random.default_rng(8).standard_normal((68, 3))
+    u /= np.linalg.norm(u, axis=1)[:, None]
+    ref = oracle.bh(pos, u, theta, 1, "f64", 1.0, 1.0, 1.0, 2.5, True)
+    ctx = ff.ff_create(ff.ff_params_default(n=68, precision="f64", count_interactions=1))
+    ff.ff_set_particles(ctx, pos, u)
+    h, f = ff.ff_dipolar_field(ctx, ff.FF_ALGO_BH, theta, True)
+    acc, pairs, opened = ff.ff_get_counts(ctx)
+    assert np.array_equal(acc, ref["nacc"]) and np.array_equal(pairs, ref["npair"])
+    assert np.array_equal(opened, ref["nopen"])
+    assert rel_err(h, ref["h"]).max() <= 1e-10 and rel_err(f, ref["f"]).max() <= 1e-10
+
+
 @pytest.mark.parametrize("leaf_max", [1, 6])
 @pytest.mark.parametrize("n", [1, 31, 33, 3001, 120011])
 def test_gradient_records_match_lists(ff, n, leaf_max):
