@@ -328,7 +328,14 @@ ff_status ff_mz_sensitivity(ff_ctx *ctx, int64_t nsteps, int64_t every, double *
 /* Waits for the context's stream and reports any error flag raised on the GPU. */
 ff_status ff_synchronize(ff_ctx *ctx);
 
-/* Tree size and interaction totals of the last Barnes-Hut evaluation (waits). */
+/*
+ * Tree size and interaction totals of the last Barnes-Hut evaluation (the
+ * totals are zero where it did not count interactions).  Waits.  A
+ * single-precision gradient without interaction counting leaves the counts to
+ * be taken when they are first asked for, here or in ff_get_counts: that call
+ * then runs one counting traversal of the gradient's tree (the time of a field
+ * evaluation's traversal), later ones copy its result.
+ */
 ff_status ff_tree_info(ff_ctx *ctx, ff_tree_info_t *out);
 
 /*
@@ -346,7 +353,9 @@ ff_status ff_get_tree(ff_ctx *ctx, uint64_t *keys, uint32_t *order, int32_t *pbe
 /*
  * Per-particle counts of the last Barnes-Hut evaluation in the caller's
  * order (host arrays of n, any may be NULL): accepted cells, exact pairs and
- * opened cells.  Needs count_interactions = 1.  Waits.
+ * opened cells.  Needs count_interactions = 1, or a Barnes-Hut gradient as the
+ * last evaluation (then the first call may run a counting traversal: see
+ * ff_tree_info).  Waits.
  */
 ff_status ff_get_counts(ff_ctx *ctx, int32_t *accepted, int32_t *pairs, int32_t *opened);
 

@@ -461,20 +461,6 @@ ff_status eval_bh(ff_ctx* c, double theta, int include_sr, bool force_counts = f
     return FF_OK;
 }
 
-// The interaction counts of a gradient's evaluation, whose walk does not split
-// its sources into cells and pairs: the counting walk on the same tree.
-template <typename R>
-void count_again(ff_ctx* c)
-{
-    Buffers& b = c->st[c->cur];
-    ffk::bh_field<R>(V<R>(b.pos), V<R>(b.u), c->n, tree_of<R>(c),
-                     field_params<R>(c, c->lazy_theta, c->lazy_sr), V<R>(c->h), V<R>(c->f),
-                     static_cast<R*>(c->esr), c->counts, c->dflags, c->work, traverse_group(c),
-                     c->sched, c->off, segs_of(c), c->stream);
-    c->counts_lazy = false;
-    c->counts_valid = true;
-}
-
 template <typename R>
 ff_status eval_ap(ff_ctx* c, int include_sr)
 {
@@ -547,6 +533,27 @@ ff_status sync_and_check(ff_ctx* c)
         const ff_status s = recover_cells(c);
         return s == FF_OK ? kRetry : s;
     }
+    return FF_OK;
+}
+
+// The interaction counts of a gradient's evaluation, whose walk does not split
+// its sources into cells and pairs: the counting walk on the same tree (which
+// writes the field, force and LJ energies too; every call that reads those
+// evaluates first).
+template <typename R>
+ff_status count_again(ff_ctx* c)
+{
+    // (an evaluation that raised a flag leaves no tree to walk)
+    ff_status s = retrying(c, [&] { return sync_and_check(c); });
+    if (s != FF_OK || !c->counts_lazy) return s;
+    Buffers& b = c->st[c->cur];
+    ffk::bh_field<R>(V<R>(b.pos), V<R>(b.u), c->n, tree_of<R>(c),
+                     field_params<R>(c, c->lazy_theta, c->lazy_sr), V<R>(c->h), V<R>(c->f),
+                     static_cast<R*>(c->esr), c->counts, c->dflags, c->work, traverse_group(c),
+                     c->sched, c->off, segs_of(c), c->stream);
+    FF_LAUNCHED(c);
+    c->counts_lazy = false;
+    c->counts_valid = true;
     return FF_OK;
 }
 
@@ -1707,11 +1714,12 @@ ff_status ff_synchronize(ff_ctx* c)
 
 ff_status ff_tree_info(ff_ctx* c, ff_tree_info_t* out)
 {
+    LaunchTally tally_(c);
     ff_status s = usable(c, true);
     if (s != FF_OK) return s;
     if (!out) return fail(c, FF_EINVAL, "out is NULL");
     if (!c->tree_valid) return fail(c, FF_ESTATE, "no Barnes-Hut tree has been built");
-    if (c->counts_lazy) count_again<float>(c);
+    if (c->counts_lazy && (s = count_again<float>(c)) != FF_OK) return s;
     if ((s = retrying(c, [&] { return sync_and_check(c); })) != FF_OK) return s;
     std::memset(out, 0, sizeof(*out));
     uint32_t nc = 0;
@@ -1825,7 +1833,7 @@ ff_status ff_get_counts(ff_ctx* c, int32_t* accepted, int32_t* pairs, int32_t* o
     LaunchTally tally_(c);
     ff_status s = usable(c, true);
     if (s != FF_OK) return s;
-    if (c->counts_lazy) count_again<float>(c);
+    if (c->counts_lazy && (s = count_again<float>(c)) != FF_OK) return s;
     if (!c->counts_valid) return fail(c, FF_ESTATE, "no interaction counts recorded (count_interactions = 0 or no BH evaluation)");
     const int64_t n = c->n;
     int32_t* stg = static_cast<int32_t*>(c->staging);

@@ -213,6 +213,33 @@ def test_gradient_records_match_lists(ff, n, leaf_max):
         assert np.array_equal(a, b)
 
 
+def test_counts_taken_after_a_gradient(ff):
+    """Without interaction counting the counts of a gradient's evaluation are taken when first
+    asked for: by either call, once, as one of the context's launches."""
+    pos, u = _gas(3001, 21)
+    res = []
+    for first in (0, 1):
+        ctx = ff.ff_create(ff.ff_params_default(n=3001))
+        ff.ff_set_particles(ctx, pos, u)
+        grad = ff.ff_energy_grad(ctx, ff.FF_ALGO_BH, 0.5, dtype=np.float32)
+        ff.ff_profile(ctx, True)
+        if first:
+            counts = ff.ff_get_counts(ctx)
+            n0 = ff.ff_profile_read(ctx)["launches"]
+            info = ff.ff_tree_info(ctx)
+            assert ff.ff_profile_read(ctx)["launches"] == n0
+        else:
+            info = ff.ff_tree_info(ctx)
+            assert ff.ff_profile_read(ctx)["launches"] == 1
+            counts = ff.ff_get_counts(ctx)
+        assert info["interactions"] == int(counts[0].sum()) + int(counts[1].sum()) > 0
+        again = ff.ff_energy_grad(ctx, ff.FF_ALGO_BH, 0.5, dtype=np.float32)
+        assert again[0] == grad[0] and np.array_equal(again[1], grad[1])
+        res.append(counts)
+    for a, b in zip(*res):
+        assert np.array_equal(a, b)
+
+
 def test_gradient_records_outgrow_their_pool(ff):
     """At a small opening angle a task's records need more chunks than the pool's first
     allocation (6000 particles, nearly all of them a source of each task: 17,600 chunks against
