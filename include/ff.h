@@ -235,9 +235,14 @@ ff_status ff_system_moments(ff_ctx *ctx, double *out, int64_t *nsteps, int32_t r
  * own particle's decisions in depth-first order), only the speed differs with
  * the workload.  This sorts the current state and builds the tree once (like
  * ff_dipolar_field with the context's theta, LJ included), then times `reps`
- * traversals for each candidate with CUDA events on the context's stream and
- * keeps the fastest (minimum over reps; ties to the earlier candidate) as the
- * context's traverse_group for later ff_step and ff_dipolar_field calls.
+ * of the context's traversals (counting interactions if it does) for each
+ * candidate with CUDA events on the context's stream and keeps the fastest
+ * (minimum over reps; ties to the earlier candidate) as the context's
+ * traverse_group for later ff_step and ff_dipolar_field calls.  One walk serves
+ * every G in double precision, with dipole-position terms, and in single
+ * precision without interaction counting up to 106,496 particles: it is timed
+ * once, every candidate gets that time, *best_group the first, and the context
+ * is left as it is.
  * groups[ngroups]: candidates (each one of 1, 2, 4, 8, 16, 32), or NULL with
  * ngroups = 0 for all six.  reps = 1 .. 100.  *best_group receives the choice;
  * ms (may be NULL) receives ngroups (6 for NULL groups) per-candidate times in
@@ -252,9 +257,9 @@ ff_status ff_tune_traversal(ff_ctx *ctx, const int32_t *groups, int32_t ngroups,
  * ff_schedule_count() is a lane group (as traverse_group) with, for the plain
  * single-precision walk (interaction counting off, no dipole-position terms),
  * its own compiled block shape: threads per block and the resident blocks per
- * SM the kernel's register budget is set for; other walks use their group's
- * default shape, and the plain single-precision walk of up to 106,496 particles
- * has one shape of its own whatever the schedule.  The traversal is persistent (as many blocks as fit), so the
+ * SM the kernel's register budget is set for; the counting walk uses its
+ * group's default shape, and the walks that serve every group (see
+ * ff_tune_traversal) have their own whatever the schedule.  The traversal is persistent (as many blocks as fit), so the
  * shape trades registers per thread against resident warps.  Every schedule
  * gives bit-identical fields and forces (in single precision each particle's
  * sources are added in depth-first order; in double precision they go in turn,
@@ -277,7 +282,8 @@ ff_status ff_set_schedule(ff_ctx *ctx, int32_t index);
  * ff_dipolar_field with the context's theta, LJ included), times `reps`
  * traversals (1 .. 100) with every schedule by CUDA events on the context's
  * stream, and keeps the fastest (minimum over reps; ties to the lower index)
- * as the context's schedule.  *best_schedule receives it; ms (may be NULL)
+ * as the context's schedule (where one walk serves every schedule it is timed
+ * once and the context left as it is, as in ff_tune_traversal).  *best_schedule receives it; ms (may be NULL)
  * receives ff_schedule_count() times in milliseconds, schedule 1 first.
  * Barnes-Hut contexts only.  Waits.
  */

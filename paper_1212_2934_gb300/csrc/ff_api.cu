@@ -1146,11 +1146,13 @@ ff_status energy_grad(ff_ctx* c, int32_t algo, double theta, double* energy, boo
 
 namespace {
 
-// Sorts and builds once, then times the traversal for each candidate: lane group
-// groups[i] with launch schedule scheds[i] (scheds may be null: the default shape).
+// Sorts and builds once, then times the traversal that the context runs (counting
+// interactions if it does) for each candidate: lane group groups[i] with launch
+// schedule scheds[i] (scheds may be null: the default shape).  Where one kernel
+// serves every candidate it is timed once, for the first (*one: nothing to choose).
 template <typename R>
 ff_status tune_traversal(ff_ctx* c, const int32_t* groups, const int32_t* scheds, int ng, int reps,
-                         float* ms_out, int* best)
+                         float* ms_out, int* best, bool* one)
 {
     ff_status s = eval_bh<R>(c, c->p.theta, 1);
     if (s != FF_OK) return s;
@@ -1158,6 +1160,9 @@ ff_status tune_traversal(ff_ctx* c, const int32_t* groups, const int32_t* scheds
     Buffers& a = c->st[c->cur];
     ffk::Tree<R> t = tree_of<R>(c);
     const ffk::FieldParams<R> fp = field_params<R>(c, c->p.theta, 1);
+    int4* counts = c->p.count_interactions ? c->counts : nullptr;
+    *one = ffk::one_walk(t, c->n, counts != nullptr);
+    const int nt = *one ? 1 : ng;
     struct Events {
         std::vector<cudaEvent_t> v;
         ~Events()
@@ -1166,15 +1171,15 @@ ff_status tune_traversal(ff_ctx* c, const int32_t* groups, const int32_t* scheds
                 if (e) cudaEventDestroy(e);
         }
     } hold;
-    hold.v.assign(2 * (size_t)ng * reps, nullptr);
+    hold.v.assign(2 * (size_t)nt * reps, nullptr);
     std::vector<cudaEvent_t>& ev = hold.v;
     for (auto& e : ev) FF_CUDA(c, cudaEventCreate(&e));
-    for (int g = 0; g < ng; ++g)
+    for (int g = 0; g < nt; ++g)
         for (int r = 0; r < reps; ++r) {
             cudaEvent_t* e = &ev[2 * ((size_t)g * reps + r)];
             cudaEventRecord(e[0], c->stream);
             ffk::bh_field<R>(V<R>(a.pos), V<R>(a.u), c->n, t, fp, V<R>(c->h), V<R>(c->f),
-                             static_cast<R*>(c->esr), nullptr, c->dflags, c->work, groups[g],
+                             static_cast<R*>(c->esr), counts, c->dflags, c->work, groups[g],
                              scheds ? scheds[g] : 0, c->off, segs_of(c), c->stream);
             cudaEventRecord(e[1], c->stream);
         }
@@ -1182,7 +1187,7 @@ ff_status tune_traversal(ff_ctx* c, const int32_t* groups, const int32_t* scheds
     s = sync_and_check(c);
     float best_ms = 0.0f;
     *best = 0;
-    for (int g = 0; g < ng && s == FF_OK; ++g) {
+    for (int g = 0; g < nt && s == FF_OK; ++g) {
         float m = 0.0f;
         for (int r = 0; r < reps; ++r) {
             float x = 0.0f;
@@ -1195,6 +1200,8 @@ ff_status tune_traversal(ff_ctx* c, const int32_t* groups, const int32_t* scheds
             *best = g;
         }
     }
+    if (ms_out)
+        for (int g = nt; g < ng && s == FF_OK; ++g) ms_out[g] = best_ms;
     return s;
 }
 
@@ -1939,14 +1946,16 @@ ff_status ff_tune_traversal(ff_ctx* c, const int32_t* groups, int32_t ngroups, i
     if (reps < 1 || reps > 100) return fail(c, FF_EINVAL, "reps must be 1 .. 100");
     if (c->p.algo != FF_ALGO_BH) return fail(c, FF_EINVAL, "the context does not use Barnes-Hut");
     int best = 0;
+    bool one = false;
     const int sched0 = c->sched;
     c->sched = 0;  // a group choice replaces a tuned launch schedule
     s = retrying(c, [&] {
-        return c->fp64 ? tune_traversal<double>(c, groups, nullptr, ngroups, reps, ms, &best)
-                       : tune_traversal<float>(c, groups, nullptr, ngroups, reps, ms, &best);
+        return c->fp64 ? tune_traversal<double>(c, groups, nullptr, ngroups, reps, ms, &best, &one)
+                       : tune_traversal<float>(c, groups, nullptr, ngroups, reps, ms, &best, &one);
     });
-    if (s != FF_OK) {
+    if (s != FF_OK || one) {
         c->sched = sched0;
+        if (s == FF_OK) *best_group = groups[best];
         return s;
     }
     if (c->p.traverse_group != groups[best] || sched0 != 0) {
@@ -1995,12 +2004,13 @@ ff_status ff_tune_schedule(ff_ctx* c, int32_t reps, int32_t* best_schedule, floa
         scheds[i] = i + 1;
     }
     int best = 0;
+    bool one = false;
     s = retrying(c, [&] {
-        return c->fp64 ? tune_traversal<double>(c, groups, scheds, ffk::kNumSchedules, reps, ms, &best)
-                       : tune_traversal<float>(c, groups, scheds, ffk::kNumSchedules, reps, ms, &best);
+        return c->fp64 ? tune_traversal<double>(c, groups, scheds, ffk::kNumSchedules, reps, ms, &best, &one)
+                       : tune_traversal<float>(c, groups, scheds, ffk::kNumSchedules, reps, ms, &best, &one);
     });
     if (s != FF_OK) return s;
-    if (c->sched != best + 1) {
+    if (!one && c->sched != best + 1) {
         c->sched = best + 1;
         drop_graphs(c);
     }

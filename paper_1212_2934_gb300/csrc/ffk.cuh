@@ -406,6 +406,18 @@ void bh_field(const vec4<R>* pos, const vec4<R>* u, int64_t n, Tree<R> t, FieldP
 // the one-lane walk.  Needs t.child; t.cap <= kWarpWalkCells (its source words hold 29-bit indices).
 constexpr int64_t kWarpWalkMax = 106496;
 constexpr int64_t kWarpWalkCells = int64_t(1) << 29;
+template <typename R>
+bool takes_warp_walk(const Tree<R>& t, int64_t n, bool counting)
+{
+    return sizeof(R) == 4 && !counting && t.child && !t.q1 && n <= kWarpWalkMax &&
+           t.cap <= kWarpWalkCells;
+}
+// Whether bh_field() runs one kernel whatever the lane group and launch schedule.
+template <typename R>
+bool one_walk(const Tree<R>& t, int64_t n, bool counting)
+{
+    return sizeof(R) == 8 || t.q1 || takes_warp_walk(t, n, counting);
+}
 void warp_walk(const float4* pos, const float4* u, int64_t n, Tree<float> t,
                FieldParams<float> fp, float4* h, float4* f, float* esr, int* flags, int* work,
                const uint32_t* off, Segs sg, cudaStream_t s);

@@ -944,7 +944,7 @@ void bh_launch(const vec4<R>* pos, const vec4<R>* u, int64_t n, Tree<R> t, Field
     if constexpr (sizeof(R) == 4 && !COUNT) {
         // few particles: a warp per task shares its reading of the tree, and no lane
         // group or launch schedule applies
-        if (t.child && !t.q1 && n <= kWarpWalkMax && t.cap <= kWarpWalkCells) {
+        if (takes_warp_walk(t, n, COUNT)) {
             warp_walk(pos, u, n, t, fp, h, f, esr, flags, work, off, sg, s);
             return;
         }

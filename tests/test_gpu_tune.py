@@ -122,3 +122,34 @@ def test_every_schedule_gives_the_same_bits(ff, prec):
         assert np.array_equal(a, b)
     with pytest.raises(ff.FFError):
         ff.ff_set_schedule(ctx, len(scheds) + 1)
+
+
+def _lattice_gas(n, seed):
+    rng = np.random.default_rng(seed)
+    m = max(2, int(np.ceil((3.1 * n) ** (1.0 / 3.0))))
+    site = rng.permutation(m ** 3)[:n]
+    q = np.stack([site // (m * m), (site // m) % m, site % m], axis=1)
+    u = rng.standard_normal((n, 3))
+    u /= np.linalg.norm(u, axis=1)[:, None]
+    return ((q + rng.uniform(-0.16, 0.16, (n, 3))) * 1.5).astype(np.float32), u.astype(np.float32)
+
+
+@pytest.mark.parametrize("n,kw,one", [(3001, {}, True), (3001, dict(precision="f64"), True),
+                                      (3001, dict(quadrupole=1), True),
+                                      (3001, dict(count_interactions=1), False),
+                                      (110011, {}, False),
+                                      (110011, dict(count_interactions=1), False)])
+def test_tuners_time_one_walk_once(ff, n, kw, one):
+    """Where one walk serves every candidate the tuners time it once and change nothing; elsewhere
+    each candidate has a time of its own."""
+    pos, u = _lattice_gas(n, 3)
+    ctx = ff.ff_create(ff.ff_params_default(n=n, **kw))
+    ff.ff_set_particles(ctx, pos, u)
+    best, ms = ff.ff_tune_traversal(ctx, reps=2)
+    assert ms[best] == min(ms.values()) and (len(set(ms.values())) == 1) == one
+    best, ms = ff.ff_tune_traversal(ctx, [8, 32], reps=1)
+    assert ms[best] == min(ms.values()) and (not one or (best == 8 and ms[8] == ms[32]))
+    best, ms = ff.ff_tune_schedule(ctx, reps=1)
+    assert ms[best] == min(ms.values()) and (len(set(ms.values())) == 1) == one
+    if kw.get("count_interactions"):
+        assert ff.ff_get_counts(ctx)[0].sum() > 0
