@@ -153,3 +153,37 @@ def test_tuners_time_one_walk_once(ff, n, kw, one):
     assert ms[best] == min(ms.values()) and (len(set(ms.values())) == 1) == one
     if kw.get("count_interactions"):
         assert ff.ff_get_counts(ctx)[0].sum() > 0
+
+
+@pytest.mark.parametrize("leaf_max", [1, 4])
+@pytest.mark.parametrize("sizes", [None, [50021, 7, 33000, 26983]])
+def test_schedules_groups_and_walks_of_large_contexts(ff, sizes, leaf_max):
+    """Above 106,496 particles the plain single-precision walk takes the context's lane group and
+    launch schedule: all of them against the counting walk, bit for bit, a ragged size, alone and
+    as a batch."""
+    n = 110011
+    assert n > 106496
+    if sizes is None:
+        pos, u = _lattice_gas(n, 8)
+    else:
+        assert sum(sizes) == n
+        pos = np.concatenate([_lattice_gas(k, 9 + k)[0] for k in sizes])
+        u = _lattice_gas(n, 8)[1]
+    out = []
+    for count in (1, 0):
+        ctx = ff.ff_create(ff.ff_params_default(n=n, leaf_max=leaf_max, count_interactions=count))
+        if sizes is not None:
+            ff.ff_set_systems(ctx, sizes)
+        ff.ff_set_particles(ctx, pos, u)
+        out.append(ff.ff_dipolar_field(ctx, ff.FF_ALGO_BH, 0.5, True))
+    h0, f0 = out[0]
+    assert np.array_equal(out[1][0], h0) and np.array_equal(out[1][1], f0)
+    for i in ff.ff_schedules():
+        ff.ff_set_schedule(ctx, i)
+        h, f = ff.ff_dipolar_field(ctx, ff.FF_ALGO_BH, 0.5, True)
+        assert np.array_equal(h, h0) and np.array_equal(f, f0), i
+    for g in ff.TRAVERSE_GROUPS:
+        best, _ = ff.ff_tune_traversal(ctx, [g], reps=1)
+        assert best == g
+        h, f = ff.ff_dipolar_field(ctx, ff.FF_ALGO_BH, 0.5, True)
+        assert np.array_equal(h, h0) and np.array_equal(f, f0), g
