@@ -300,9 +300,10 @@ struct ChunkWriter {
 };
 
 // pair_r2() with the last operation left for the compiler to fuse (it can only be
-// the same one): written out, it costs the one-lane walk a spilled word and, with
-// leaves of several particles, 1 % (field of 1,500,032 particles, leaf_max 8, theta
-// 0.6: 8.56 ms, written out 8.66).
+// the same one), for the particles of opened leaves: written out there, it cost
+// fields with leaves of several particles 1 % (1,048,576 particles, leaf_max 8, theta
+// 0.6: 5.69 ms, so 5.65).  In the cell's own r^2 it is the other way round
+// (150,000 particles, leaf_max 1, theta 0.4: 1.682 ms written out, 1.695 so).
 template <typename R>
 __device__ __forceinline__ R lane_r2(R rx, R ry, R rz)
 {
@@ -349,7 +350,7 @@ __device__ __forceinline__ void bh_task1(int task, const vec4<R>* __restrict__ p
         // the separation serves the opening test (each component rounded once
         // either way) and the pair terms
         const R rx = rsub(xk.x, c.x), ry = rsub(xk.y, c.y), rz = rsub(xk.z, c.z);
-        const R r2 = QUAD ? rx * rx + ry * ry + rz * rz : lane_r2(rx, ry, rz);
+        const R r2 = QUAD ? rx * rx + ry * ry + rz * rz : pair_r2(rx, ry, rz);
         const bool out1 = single && !inside;
         // A one-particle leaf adds the same dipole term whether accepted or
         // summed as a pair; the two differ only by the LJ term, which is zero
