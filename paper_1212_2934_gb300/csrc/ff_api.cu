@@ -237,6 +237,7 @@ ffk::Tree<R> tree_of(ff_ctx* c)
     // the same cutoff as field_params' rcut (the opening rule's LJ cut)
     const bool lj_on = c->p.lj_eps != 0.0 && c->p.lj_rcut > 0.0;
     t.rcut = lj_on ? (R)c->p.lj_rcut : R(0);
+    t.leaf_max = c->p.leaf_max;
     return t;
 }
 

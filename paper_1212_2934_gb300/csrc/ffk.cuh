@@ -172,6 +172,7 @@ struct Tree {
     vec4<R>* q1 = nullptr;
     vec4<R>* q2 = nullptr;
     R rcut = R(0);       // LJ cutoff of the opening rule (0: LJ off)
+    int leaf_max;        // most particles of a leaf above the deepest level
 };
 
 // Square of the distance from a cell's centre beyond which a particle is

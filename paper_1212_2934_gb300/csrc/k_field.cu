@@ -96,9 +96,8 @@ constexpr int kTraverseCarveout = FFK_TRAVERSE_CARVEOUT;
 // for the whole walk without spills.  The plain FP32 walk is lean enough for
 // 128 x 12 (40 registers, 48 warps) with a few spilled words, and measures
 // slightly faster so; the other walks keep 10 blocks.  The walk with
-// dipole-position terms gains from more registers (54 a thread with 8 blocks asked
-// for, 36 warps an SM) only while all of its tasks are resident at once, where
-// fewer warps cost nothing: see bh_launch().
+// dipole-position terms also has a shape with more registers (54 a thread with 8
+// blocks asked for, 36 warps an SM): see quad_few_warps().
 #ifndef FFK_BH_THREADS
 #define FFK_BH_THREADS 128
 #endif
@@ -911,9 +910,26 @@ __global__ void __launch_bounds__(32 * kAp2Warps, 2) k_ap2(const float4* __restr
 
 }  // namespace
 
-// RESIDENT: only where every task finds a warp at once (else false, and no launch).
+// Whether the walk with dipole-position terms takes the shape with more registers
+// and `resident` warps at once (54 registers, 36 warps on each of 152 SMs).  While
+// every task has a warp at once, or all but a few that start as the first end (to
+// 182,080 particles), fewer warps cost nothing.  Beyond, the 40 warps of the other
+// shape hide more of its loads, except at small opening angles with one-particle
+// leaves, where a task does more arithmetic a load (but not up to 1.4 waves of
+// warps, where what the second wave holds runs alone).  Field calls, ms with 10 / 8
+// blocks: 131,071 particles at theta 0.7 0.976 / 0.940; 180,000 at 0.4 3.22 / 3.09;
+// 200,000 at 0.5 2.10 / 2.33; 1,048,576 at 0.7 4.36 / 4.65, at 0.5 9.47 / 9.79; at 0.4
+// 192,000 3.33 / 3.70, 288,000 5.17 / 4.97, 400,000 6.77 / 6.60, 700,000 11.8 / 11.5
+// (leaf_max 2: 300,000 5.16 / 5.27); at 0.3 400,000 15.4 / 14.1.
+bool quad_few_warps(int64_t ntask, int64_t resident, double theta2, int leaf_max)
+{
+    if (25 * ntask <= 26 * resident) return true;
+    return theta2 < 0.2 && leaf_max == 1 && 5 * ntask > 7 * resident;
+}
+
+// FEW: only where quad_few_warps() (else false, and no launch).
 template <typename R, bool COUNT, int G, bool QUAD = false, int THREADS = kBhThreads,
-          int MINB = bh_min_blocks<R, COUNT, QUAD>(), bool RESIDENT = false>
+          int MINB = bh_min_blocks<R, COUNT, QUAD>(), bool FEW = false>
 bool bh_launch_g(const vec4<R>* pos, const vec4<R>* u, int64_t n, Tree<R> t, FieldParams<R> fp,
                  vec4<R>* h, vec4<R>* f, R* esr, int4* counts, int* flags, int* work,
                  const uint32_t* off, Segs sg, cudaStream_t s)
@@ -930,7 +946,9 @@ bool bh_launch_g(const vec4<R>* pos, const vec4<R>* u, int64_t n, Tree<R> t, Fie
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, THREADS, 0);
         return per_sm;
     });
-    if (RESIDENT && (n + 31) / 32 > (int64_t)g.blocks * (THREADS / 32)) return false;
+    if (FEW && !quad_few_warps((n + 31) / 32, (int64_t)g.blocks * (THREADS / 32),
+                               (double)fp.theta2, t.leaf_max))
+        return false;
     cudaMemsetAsync(work, 0, sizeof(int) * g.nseg, s);
     kern<<<g.blocks, THREADS, 0, s>>>(pos, u, (int)n, t, fp, h, f, esr, counts, flags, work,
                                       g.nseg, off, sg);
@@ -980,12 +998,8 @@ void bh_launch(const vec4<R>* pos, const vec4<R>* u, int64_t n, Tree<R> t, Field
     } else {
     if (sched >= 1 && sched <= kNumSchedules) group = kSchedules[sched - 1].group;
     if (t.q1) {
-        // the dipole-position terms are evaluated by the one-lane walk only.  While every
-        // task has a warp at once (to 175,104 particles: 54 registers, 36 warps on each
-        // of 152 SMs) it takes the shape with more registers; beyond, the 40 warps of the
-        // other hide more of its loads.  Field calls, ms with 10 / 8 blocks: 131,071
-        // particles at theta 0.7 0.976 / 0.940; 200,000 at 0.5 2.13 / 2.33; 1,048,576 at
-        // 0.7 4.47 / 4.65, at 0.5 9.60 / 9.77.
+        // the dipole-position terms are evaluated by the one-lane walk only, in one of
+        // two shapes (quad_few_warps)
         if (!bh_launch_g<R, COUNT, 1, true, kBhThreads, kBhMinBlocksQuadFew, true>(
                 pos, u, n, t, fp, h, f, esr, counts, flags, work, off, sg, s))
             bh_launch_g<R, COUNT, 1, true>(pos, u, n, t, fp, h, f, esr, counts, flags, work, off,

@@ -52,10 +52,13 @@ def test_quadrupole_matches_oracle(ff, ora, prec, leaf_max):
     assert np.array_equal(acc, ref["nacc"]) and np.array_equal(opened, ref["nopen"])
 
 
-@pytest.mark.parametrize("n", [150011, 175104, 175105, 200003])
-def test_quadrupole_on_both_sides_of_the_shape_switch(ff, ora, n):
-    """The walk has two block shapes, chosen by whether all of its tasks are resident at once
-    (175,104 particles on 152 SMs): both against the oracle, at the plain bar."""
+@pytest.mark.parametrize("n,theta,leaf_max", [(150011, 0.7, 1), (182080, 0.7, 1), (182081, 0.7, 1),
+                                              (200003, 0.7, 1), (200003, 0.4, 1), (245120, 0.4, 1),
+                                              (245121, 0.4, 1), (260003, 0.4, 1), (260003, 0.4, 2)])
+def test_quadrupole_on_both_sides_of_the_shape_switch(ff, ora, n, theta, leaf_max):
+    """The walk has two block shapes, chosen by how many of its tasks are resident at once (the
+    lines lie at 182,080 and 245,120 particles on 152 SMs), the opening angle and the leaves: both against the oracle,
+    at the plain bar."""
     rng = np.random.default_rng(n)
     m = int(np.ceil((3.1 * n) ** (1.0 / 3.0)))
     site = rng.permutation(m ** 3)[:n]
@@ -63,12 +66,12 @@ def test_quadrupole_on_both_sides_of_the_shape_switch(ff, ora, n):
     pos = ((q + rng.uniform(-0.16, 0.16, (n, 3))) * 1.5).astype(np.float32)
     u = rng.standard_normal((n, 3))
     u = (u / np.linalg.norm(u, axis=1)[:, None]).astype(np.float32)
-    ctx = ff.ff_create(ff.ff_params_default(n=n, quadrupole=1))
+    ctx = ff.ff_create(ff.ff_params_default(n=n, quadrupole=1, leaf_max=leaf_max))
     ff.ff_set_particles(ctx, pos, u)
-    h, f = ff.ff_dipolar_field(ctx, ff.FF_ALGO_BH, 0.7, True)
+    h, f = ff.ff_dipolar_field(ctx, ff.FF_ALGO_BH, theta, True)
     sel = np.concatenate([rng.integers(0, n, 200), np.arange(n - 40, n)])
-    ref = ora.bh(pos.astype(np.float64), u.astype(np.float64), 0.7, 1, "f32", 1.0, 1.0, 1.0, 2.5,
-                 True, only=np.unique(sel), quad=True)
+    ref = ora.bh(pos.astype(np.float64), u.astype(np.float64), theta, leaf_max, "f32", 1.0, 1.0,
+                 1.0, 2.5, True, only=np.unique(sel), quad=True)
     sel = np.unique(sel)
     assert rel_err(h[sel], ref["h"][sel]).max() <= 1e-5
     assert rel_err(f[sel], ref["f"][sel]).max() <= 1e-5
