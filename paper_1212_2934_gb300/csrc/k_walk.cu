@@ -18,8 +18,8 @@
 // the other, so fields and forces have the bits of the one-lane walk.
 //
 // Measured on GB300 (volume fraction 0.05, theta 0.5), one-lane walk -> this:
-//   n = 1,000  0.383 -> 0.167 ms     n = 65,536   0.653 -> 0.575 ms
-//   n = 16,384 0.547 -> 0.316 ms     n = 100,000  0.742 -> 0.721 ms
+//   n = 1,000  0.409 -> 0.157 ms     n = 65,536   0.647 -> 0.566 ms
+//   n = 16,384 0.525 -> 0.313 ms     n = 100,000  0.741 -> 0.716 ms
 // and 4.85 -> 5.45 ms at n = 1,048,576, where the one-lane walk has enough
 // warps to hide its loads and this one adds every source of a task in all of
 // its lanes (1784 of which a lane uses 813): the summing is bound by the FP32

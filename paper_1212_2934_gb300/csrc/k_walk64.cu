@@ -14,9 +14,9 @@
 //
 // A particle's sums depend on its own list alone (four partial sums added in a
 // fixed order), not on its neighbours in the warp.  Measured on GB300 (volume
-// fraction 0.05, theta 0.5), one-lane walk -> this: n = 4,096 1.52 -> 0.39 ms,
-// 16,384 2.00 -> 1.21, 50,000 5.68 -> 3.26, 262,144 29.9 -> 20.0 (the last and
-// the 16,384 with lists of 320); the FP64 units are 87 % busy at n = 100,000.
+// fraction 0.05, theta 0.5), one-lane walk -> this: n = 4,096 1.53 -> 0.39 ms,
+// 16,384 1.98 -> 1.14, 50,000 5.57 -> 3.24, 100,000 12.0 -> 6.87, 262,144 29.9 ->
+// 19.4; the FP64 units are 86 % busy at n = 100,000.
 #include "walk_stack.cuh"
 
 namespace ffk {
